@@ -111,27 +111,30 @@ __device__ __forceinline__ unsigned chain_track_fp64(float (&pf)[6], float (&Cf)
                                                      int64_t hc_stride, const ChainLoc &l3,
                                                      const ChainLoc &l6) {
   double p[6], C[21];
-  for (int c = 0; c < 6; ++c) p[c] = pf[c];
-  for (int e = 0; e < 21; ++e) C[e] = Cf[e];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) p[c] = f64::from_float(pf[c]);
+#pragma unroll
+  for (int e = 0; e < 21; ++e) C[e] = f64::from_float(Cf[e]);
+  const double q = f64::from_float(qf), b = f64::from_float(bz);
   unsigned st = 0;
   HitCursor cur(hits, hit_stride, hitcovs, hc_stride, l3, l6);
   for (int l = 0; l < L; ++l, cur.next_layer()) {
     LayerHit h;
     cur.load(h, kinds[l]);
-    double hc[6], rcos;
-    bool shrink;
-    for (int c = 0; c < 6; ++c) hc[c] = h.hc[c];
+    double hc[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) hc[c] = f64::from_float(h.hc[c]);
+    const double hx = f64::from_float(h.hx), hy = f64::from_float(h.hy);
+    const double ps = f64::from_float(pos[l]);
     if (kinds[l] == kP2z)
-      st |= p2z_step_t<double, kStandard>(p, C, (double)qf, (double)bz, (double)pos[l],
-                                          (double)h.hx, (double)h.hy, hc[0], hc[1], hc[2],
-                                          shrink);
+      st |= f64::p2z_step(p, C, q, b, ps, hx, hy, hc[0], hc[1], hc[2]);
     else
-      st |= p2r_step_t<double, kStandard>(p, C, (double)qf, (double)bz, (double)pos[l],
-                                          (double)h.hx, (double)h.hy, (double)h.hz, hc, shrink,
-                                          rcos);
+      st |= f64::p2r_step(p, C, q, b, ps, hx, hy, f64::from_float(h.hz), hc);
   }
-  for (int c = 0; c < 6; ++c) pf[c] = (float)p[c];
-  for (int e = 0; e < 21; ++e) Cf[e] = (float)C[e];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) pf[c] = f64::to_float(p[c]);
+#pragma unroll
+  for (int e = 0; e < 21; ++e) Cf[e] = f64::to_float(C[e]);
   return st;
 }
 

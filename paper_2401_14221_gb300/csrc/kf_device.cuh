@@ -5,10 +5,10 @@
 // (KalmanUpdate).  The paper gives no formulas; this file implements the
 // exact helix in a uniform field bz, its transport Jacobian and the linear
 // Kalman update, in registers, one track per thread.  The arithmetic is
-// written once for a number type T (kf_num.cuh): float is the bulk path,
-// double serves the FP64 variants and the FP64 redo of ill-conditioned
-// tracks.  Every operation is explicitly rounded, so a track's result does
-// not depend on which kernel computes it.
+// written in terms of a number type T (kf_num.cuh): float, the bulk path.  The
+// FP64 variant and the FP64 redo of ill-conditioned tracks have a step of
+// their own (kf_fp64.cuh).  Every operation is explicitly rounded, so a
+// track's result does not depend on which kernel computes it.
 //
 // Design notes (what differs from a textbook transcription):
 //  * The helix uses the half-angle form (chord = 2 sin(h)/omega with
@@ -30,16 +30,12 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "kf_fp64.cuh"
 #include "kf_num.cuh"
 
 namespace kf {
 
 using namespace num;
-
-constexpr unsigned kNoIntersect = 1u;
-constexpr unsigned kSNotPD = 2u;
-constexpr unsigned kBadK = 4u;
-constexpr unsigned kNonFinite = 8u;
 
 // Update variants (the KF_* precision values of the C ABI).
 enum Variant : int {
@@ -77,16 +73,6 @@ struct Consts<float> {
   static constexpr double dsinc_series = 0.25;  // below: Taylor series for S'(h)
 };
 
-template <>
-struct Consts<double> {
-  static constexpr double alpha = 0.299792458e-2;
-  static constexpr double pi = 3.141592653589793;
-  static constexpr double two_pi_hi = 6.283185307179586;
-  static constexpr double two_pi_lo = 2.4492935982947064e-16;
-  static constexpr double inv_two_pi = 0.15915494309189535;
-  static constexpr double dsinc_series = 0.05;
-};
-
 template <class T>
 using K_ = Consts<scalar_t<T>>;
 
@@ -94,11 +80,6 @@ using K_ = Consts<scalar_t<T>>;
 template <class T, class FA, class FB>
 __device__ __forceinline__ T choose(mask_t<T> m, FA &&a, FB &&b) {
   return m ? a() : b();
-}
-
-// Packed lower-triangular index of a symmetric matrix element.
-__host__ __device__ constexpr int tri(int i, int j) {
-  return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i;
 }
 
 constexpr uint64_t bit(int i, int j) { return 1ull << (i * 6 + j); }
@@ -734,31 +715,30 @@ __device__ __forceinline__ stat_t<T> p2r_step_t(T (&p)[6], T (&C)[21], T qf, T b
   return step_status<T>(bad, p[3]);
 }
 
-// Run a T = double step on float registers (convert in and out).  Kept out
-// of line so that the float path's register allocation does not carry it.
+// Run the double-precision step on float registers (convert in and out).
 template <int KIND>
-__device__ __noinline__ unsigned step_in_double(float (&p)[6], float (&C)[21], float qf, float bz,
-                                                float surf, float hx, float hy, float hz,
-                                                const float (&hc)[6]) {
-  double dp[6], dC[21], dhc[6], cinc;
-  bool shrink;
+__device__ __forceinline__ unsigned step_in_double(float (&p)[6], float (&C)[21], float qf,
+                                                   float bz, float surf, float hx, float hy,
+                                                   float hz, const float (&hc)[6]) {
+  double dp[6], dC[21], dhc[6];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) dp[i] = p[i];
+  for (int i = 0; i < 6; ++i) dp[i] = f64::from_float(p[i]);
 #pragma unroll
-  for (int e = 0; e < 21; ++e) dC[e] = C[e];
+  for (int e = 0; e < 21; ++e) dC[e] = f64::from_float(C[e]);
 #pragma unroll
-  for (int i = 0; i < 6; ++i) dhc[i] = hc[i];
+  for (int i = 0; i < 6; ++i) dhc[i] = f64::from_float(hc[i]);
+  const double q = f64::from_float(qf), b = f64::from_float(bz), sf = f64::from_float(surf);
+  const double x = f64::from_float(hx), y = f64::from_float(hy);
   unsigned st;
   if (KIND == kP2z)
-    st = p2z_step_t<double, kStandard>(dp, dC, qf, bz, surf, hx, hy, dhc[0], dhc[1], dhc[2],
-                                       shrink);
+    st = f64::p2z_step(dp, dC, q, b, sf, x, y, dhc[0], dhc[1], dhc[2]);
   else
-    st = p2r_step_t<double, kStandard>(dp, dC, qf, bz, surf, hx, hy, hz, dhc, shrink, cinc);
+    st = f64::p2r_step(dp, dC, q, b, sf, x, y, f64::from_float(hz), dhc);
   if (!(st & kNoIntersect)) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) p[i] = (float)dp[i];
+    for (int i = 0; i < 6; ++i) p[i] = f64::to_float(dp[i]);
 #pragma unroll
-    for (int e = 0; e < 21; ++e) C[e] = (float)dC[e];
+    for (int e = 0; e < 21; ++e) C[e] = f64::to_float(dC[e]);
   }
   return st;
 }

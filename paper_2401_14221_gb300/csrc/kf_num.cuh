@@ -1,8 +1,9 @@
 // kf_num.cuh -- the number types of the per-track arithmetic, with every
 // rounding written out.
 //
-// The step is written once (kf_device.cuh) for a number type T: float (the
-// FP32 bulk path) or double (the FP64 variants and redo passes).  Every
+// The step (kf_device.cuh) is written in terms of a number type T: float,
+// the FP32 bulk path.  (The double-precision step has algebra of its own,
+// kf_fp64.cuh.)  Every
 // operation is an explicit, individually rounded IEEE operation: a product
 // and a sum are fused only where the source says fma_, never by the
 // compiler.  So every kernel that runs the same source on the same inputs
@@ -20,6 +21,18 @@
 #include <cuda_runtime.h>
 
 namespace kf {
+
+// Status bits of a track (the KF_* status values of the C ABI).
+constexpr unsigned kNoIntersect = 1u;
+constexpr unsigned kSNotPD = 2u;
+constexpr unsigned kBadK = 4u;
+constexpr unsigned kNonFinite = 8u;
+
+// Packed lower-triangular index of a symmetric matrix element.
+__host__ __device__ constexpr int tri(int i, int j) {
+  return i >= j ? i * (i + 1) / 2 + j : j * (j + 1) / 2 + i;
+}
+
 namespace num {
 
 // ================================================================== float
@@ -45,28 +58,6 @@ __device__ __forceinline__ bool gt_(float a, float b) { return a > b; }
 __device__ __forceinline__ bool ge_(float a, float b) { return a >= b; }
 __device__ __forceinline__ float sel_(bool m, float a, float b) { return m ? a : b; }
 __device__ __forceinline__ bool finite_(float a) { return isfinite(a); }
-
-// ================================================================= double
-__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ double neg_(double a) { return -a; }
-__device__ __forceinline__ double abs_(double a) { return fabs(a); }
-__device__ __forceinline__ double sqrt_(double a) { return sqrt(a); }
-__device__ __forceinline__ double rsqrt_(double a) { return rsqrt(a); }
-__device__ __forceinline__ double rint_(double a) { return rint(a); }
-__device__ __forceinline__ double div_(double a, double b) { return __ddiv_rn(a, b); }
-__device__ __forceinline__ double rcp_(double b) { return __ddiv_rn(1.0, b); }
-__device__ __forceinline__ double atan2_(double y, double x) { return atan2(y, x); }
-__device__ __forceinline__ void sincos_(double x, double *s, double *c) { sincos(x, s, c); }
-
-__device__ __forceinline__ bool lt_(double a, double b) { return a < b; }
-__device__ __forceinline__ bool le_(double a, double b) { return a <= b; }
-__device__ __forceinline__ bool gt_(double a, double b) { return a > b; }
-__device__ __forceinline__ bool ge_(double a, double b) { return a >= b; }
-__device__ __forceinline__ double sel_(bool m, double a, double b) { return m ? a : b; }
-__device__ __forceinline__ bool finite_(double a) { return isfinite(a); }
 
 // Masks and status words of the scalar types.
 __device__ __forceinline__ bool all_(bool m) { return m; }
@@ -189,18 +180,12 @@ template <> struct Traits<float> {
   using stat = unsigned;
   using scalar = float;
 };
-template <> struct Traits<double> {
-  using mask = bool;
-  using stat = unsigned;
-  using scalar = double;
-};
 template <class T> using mask_t = typename Traits<T>::mask;
 template <class T> using stat_t = typename Traits<T>::stat;
 template <class T> using scalar_t = typename Traits<T>::scalar;
 
 template <class T> __device__ __forceinline__ T cst(double v);
 template <> __device__ __forceinline__ float cst<float>(double v) { return (float)v; }
-template <> __device__ __forceinline__ double cst<double>(double v) { return v; }
 
 // A status word with `b` set where m holds.
 template <class T>

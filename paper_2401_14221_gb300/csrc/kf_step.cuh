@@ -50,31 +50,17 @@ __device__ __forceinline__ unsigned redo_track_fp64(const StepArgs &a, int64_t i
     b3 = blk * 3 * W + r;
     s = W;
   }
-  double p[6], C[21], hc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, cinc;
-  bool shrink;
+  float pf[6], Cf[21], hc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-  for (int c = 0; c < 6; ++c) p[c] = a.state_in[b6 + c * s];
+  for (int c = 0; c < 6; ++c) pf[c] = a.state_in[b6 + c * s];
 #pragma unroll
-  for (int e = 0; e < 21; ++e) C[e] = a.cov_in[b21 + e * s];
+  for (int e = 0; e < 21; ++e) Cf[e] = a.cov_in[b21 + e * s];
   constexpr int nhc = KIND == kP2z ? 3 : 6;
 #pragma unroll
   for (int c = 0; c < nhc; ++c) hc[c] = a.hitcov[b6 + c * s];
-  const double qf = a.charge[i];
-  const double surf = a.surf[a.surf_per_track ? i : 0];
-  const double hx = a.hit[b3], hy = a.hit[b3 + s];
-  unsigned st;
-  if (KIND == kP2z)
-    st = p2z_step_t<double, kStandard>(p, C, qf, (double)a.bz, surf, hx, hy, hc[0], hc[1], hc[2],
-                                       shrink);
-  else
-    st = p2r_step_t<double, kStandard>(p, C, qf, (double)a.bz, surf, hx, hy,
-                                       (double)a.hit[b3 + 2 * s], hc, shrink, cinc);
-  // exact when the track was not propagated (float -> double -> float)
-  float pf[6], Cf[21];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) pf[c] = (float)p[c];
-#pragma unroll
-  for (int e = 0; e < 21; ++e) Cf[e] = (float)C[e];
+  unsigned st = step_in_double<KIND>(pf, Cf, (float)a.charge[i], a.bz,
+                                     a.surf[a.surf_per_track ? i : 0], a.hit[b3], a.hit[b3 + s],
+                                     KIND == kP2z ? 0.0f : a.hit[b3 + 2 * s], hc);
   st |= finite_status(pf, Cf);
 #pragma unroll
   for (int c = 0; c < 6; ++c) __stcs(a.state_out + b6 + c * s, pf[c]);

@@ -36,19 +36,16 @@ __device__ __forceinline__ Loc locate(int64_t i, int64_t n, int32_t soa, int32_t
 }
 
 // Load track i: state, and the covariance decoded from sigma / rho.
-template <class T>
 __device__ __forceinline__ void load_compressed(const CompressedArgs &a, const Loc &l6,
-                                                const RhoLoc &lr, T (&p)[6], T (&C)[21]) {
-  float sg[6], Cf[21];
+                                                const RhoLoc &lr, float (&p)[6], float (&C)[21]) {
+  float sg[6];
   Rho rh;
 #pragma unroll
   for (int c = 0; c < 6; ++c) p[c] = __ldg(a.state_in + l6.base + c * l6.stride);
 #pragma unroll
   for (int c = 0; c < 6; ++c) sg[c] = __ldg(a.sigma_in + l6.base + c * l6.stride);
   load_rho(a.rho_in, lr, rh);
-  decode_cov(sg, rh, Cf);
-#pragma unroll
-  for (int e = 0; e < 21; ++e) C[e] = T(Cf[e]);
+  decode_cov(sg, rh, C);
 }
 
 // Encode and store track i's result; a track that was not propagated gets
@@ -132,27 +129,15 @@ __global__ void __launch_bounds__(kRedoThreads)
     const Loc l6 = locate<6>(i, a.n, a.soa, a.lw);
     const RhoLoc lr = locate_rho(i, a.n, a.soa, a.lw);
     const Loc l3 = locate<3>(i, a.n, a.soa, a.lw);
-    double p[6], C[21], hc[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, cinc;
-    bool shrink;
-    load_compressed(a, l6, lr, p, C);
+    float pf[6], Cf[21], hc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    load_compressed(a, l6, lr, pf, Cf);
     constexpr int nhc = KIND == kP2z ? 3 : 6;
 #pragma unroll
     for (int c = 0; c < nhc; ++c) hc[c] = a.hitcov[l6.base + c * l6.stride];
-    const double qf = a.charge[i];
-    const double surf = a.surf[a.surf_per_track ? i : 0];
-    const double hx = a.hit[l3.base], hy = a.hit[l3.base + l3.stride];
-    unsigned st;
-    if (KIND == kP2z)
-      st = p2z_step_t<double, kStandard>(p, C, qf, (double)a.bz, surf, hx, hy, hc[0], hc[1],
-                                         hc[2], shrink);
-    else
-      st = p2r_step_t<double, kStandard>(p, C, qf, (double)a.bz, surf, hx, hy,
-                                         (double)a.hit[l3.base + 2 * l3.stride], hc, shrink, cinc);
-    float pf[6], Cf[21];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) pf[c] = (float)p[c];
-#pragma unroll
-    for (int e = 0; e < 21; ++e) Cf[e] = (float)C[e];
+    unsigned st = step_in_double<KIND>(pf, Cf, (float)a.charge[i], a.bz,
+                                       a.surf[a.surf_per_track ? i : 0], a.hit[l3.base],
+                                       a.hit[l3.base + l3.stride],
+                                       KIND == kP2z ? 0.0f : a.hit[l3.base + 2 * l3.stride], hc);
     st |= finite_status(pf, Cf);
     store_compressed(a, l6, lr, pf, Cf, st);
     a.status[i] = (uint8_t)st;
