@@ -582,10 +582,8 @@ int kf_server_destroy(kf_server *s);
  * this process (a tuning knob; the results are the same, bit for bit):
  *   KF_STEP_AUTO    (default) the autotuner's choice where it has one, else
  *                   the direct kernel in 128-thread CTAs (on GB300 it leads
- *                   or ties the staged kernel from 240,000 to 3.84 M tracks
- *                   and at every layout measured), and for the FP64-pipe-
- *                   bound variants (KF_FP64_UPDATE, KF_FP64) the staged
- *                   kernel at 2 CTAs/SM where it applies;
+ *                   or ties the staged kernel from 2,000 to 3.84 M tracks, at
+ *                   every layout and for every variant measured);
  *   KF_STEP_DIRECT  one thread per track with direct global loads (any
  *                   layout), 128-thread CTAs;
  *   KF_STEP_STAGED  a persistent kernel in which a producer warp streams

@@ -469,32 +469,39 @@ __device__ __forceinline__ void kalman_update_body(T (&p)[6], T (&C)[21], const 
 }
 
 // The standard form with S^-1, K and C'' in double from float inputs (the
-// kFP64Update variant).
+// kFP64Update variant).  The FP64 pipe bounds it, so as in kf_fp64.cuh the
+// floats are converted by shifts, the reciprocals come from FP32 seeds, and
+// the measured columns are K V (C'' H^T = K V cancels no digits), which needs
+// no S^-1 V: 73 FP64 instructions a p2r track where the conversions, two
+// library divisions and the U (S^-1 V) form took about 145 (960,000 p2r
+// tracks 250 -> 134 us).
 template <int SKIP, int M1, bool UNIT0>
 __device__ __forceinline__ bool kalman_update_f64(float (&p)[6], float (&C)[21],
-                                                  const float (&U0)[6], const float (&U1)[6],
-                                                  float S00, float S01, float S11, float h0,
-                                                  float V00, float V01, float V11, float r0,
-                                                  float r1) {
-  const double dS00 = S00, dS01 = S01, dS11 = S11;
-  const double det = __fma_rn(dS00, dS11, __dmul_rn(-dS01, dS01));
-  if (!(dS00 > 0.0) || !(det > 0.0)) return true;
-  const double inv = __ddiv_rn(1.0, det);
-  const double Si00 = __dmul_rn(dS11, inv), Si01 = __dmul_rn(-dS01, inv),
-               Si11 = __dmul_rn(dS00, inv);
-  double K0[6], K1[6];
+                                                  const float (&U0f)[6], const float (&U1f)[6],
+                                                  float S00f, float S01f, float S11f, float h0,
+                                                  float V00f, float V01f, float V11f, float r0f,
+                                                  float r1f) {
+  using f64::from_float;
+  using f64::to_float;
+  const double S00 = from_float(S00f), S01 = from_float(S01f), S11 = from_float(S11f);
+  const double det = __fma_rn(S00, S11, -__dmul_rn(S01, S01));
+  if (!(S00f > 0.0f) || !f64::gt0(det)) return true;
+  const double inv = f64::rcp(det);
+  const double Si00 = __dmul_rn(S11, inv), Si01 = -__dmul_rn(S01, inv), Si11 = __dmul_rn(S00, inv);
+  const double V00 = from_float(V00f), V01 = from_float(V01f), V11 = from_float(V11f);
+  const double r0 = from_float(r0f), r1 = from_float(r1f);
+  const double ih0 = UNIT0 ? 1.0 : f64::rcp(from_float(h0));
+  const double W00 = UNIT0 ? V00 : __dmul_rn(V00, ih0), W01 = UNIT0 ? V01 : __dmul_rn(V01, ih0);
+  double K0[6], K1[6], U0[6], U1[6];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     if (i == SKIP) continue;
-    K0[i] = __fma_rn((double)U0[i], Si00, __dmul_rn((double)U1[i], Si01));
-    K1[i] = __fma_rn((double)U0[i], Si01, __dmul_rn((double)U1[i], Si11));
-    p[i] = (float)__fma_rn(K0[i], (double)r0, __fma_rn(K1[i], (double)r1, (double)p[i]));
+    U0[i] = from_float(U0f[i]);
+    U1[i] = from_float(U1f[i]);
+    K0[i] = __fma_rn(U0[i], Si00, __dmul_rn(U1[i], Si01));
+    K1[i] = __fma_rn(U0[i], Si01, __dmul_rn(U1[i], Si11));
+    p[i] = to_float(__fma_rn(K0[i], r0, __fma_rn(K1[i], r1, from_float(p[i]))));
   }
-  const double G00 = __fma_rn(Si00, V00, __dmul_rn(Si01, V01));
-  const double G01 = __fma_rn(Si00, V01, __dmul_rn(Si01, V11));
-  const double G10 = __fma_rn(Si01, V00, __dmul_rn(Si11, V01));
-  const double G11 = __fma_rn(Si01, V01, __dmul_rn(Si11, V11));
-  const double ih0 = UNIT0 ? 1.0 : __ddiv_rn(1.0, (double)h0);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     if (i == SKIP) continue;
@@ -505,13 +512,12 @@ __device__ __forceinline__ bool kalman_update_f64(float (&p)[6], float (&C)[21],
       double v;
       if (mm || im) {
         const int r = mm ? i : m, c = mm ? m : i;  // row r, measured column c
-        const double g0 = __fma_rn((double)U0[r], G00, __dmul_rn((double)U1[r], G10));
-        v = (c == 0) ? (UNIT0 ? g0 : __dmul_rn(g0, ih0))
-                     : __fma_rn((double)U0[r], G01, __dmul_rn((double)U1[r], G11));
+        v = (c == 0) ? __fma_rn(K0[r], W00, __dmul_rn(K1[r], W01))
+                     : __fma_rn(K0[r], V01, __dmul_rn(K1[r], V11));
       } else {  // C' - K0 U0^T - K1 U1^T, two fused steps
-        v = __fma_rn(-K0[i], (double)U0[m], __fma_rn(-K1[i], (double)U1[m], (double)C[tri(i, m)]));
+        v = __fma_rn(-K0[i], U0[m], __fma_rn(-K1[i], U1[m], from_float(C[tri(i, m)])));
       }
-      C[tri(i, m)] = (float)v;
+      C[tri(i, m)] = to_float(v);
     }
   }
   return false;

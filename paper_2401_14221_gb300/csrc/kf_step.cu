@@ -295,14 +295,13 @@ static int launch_step_main(int kind, int precision, const StepArgs &a, cudaStre
   // The staged kernel copies whole tiles of device memory with 16-byte-
   // aligned bulk copies: any AoSoA layout, SoA when n is a multiple of 4.
   const bool staged_ok = !plain_loads && (!a.soa || (a.n & 3) == 0);
-  // KF_FP64_UPDATE is bound by GB300's FP64 pipe, where the staged kernel's
-  // decoupled loads help (960,000 p2r tracks: 262 us staged at 2 CTAs/SM
-  // against 300 us direct).  KF_FP64 needs 150 registers, which the staged
-  // kernel's 96 spill (1,000,000 tracks, direct against staged: p2r 663 and
-  // 681 us, p2z 463 and 464; 30,000: 40 and 50, 29 and 35; 2,000: 17 and 30,
-  // 12 and 21).
-  const bool staged = precision == KF_FP64_UPDATE && staged_ok;
-  LaunchConfig cfg{staged ? KF_STEP_STAGED : KF_STEP_DIRECT, kDirectThreads, 2};
+  // The variants bound by the FP64 pipe lead as direct kernels too (direct
+  // against the staged kernel's best shape, AoSoA64).  FP64 update: 1,000,000
+  // tracks p2r 140 and 147 us, p2z 130 and 137; 30,000: 9.6 and 12.5, 9.6 and
+  // 11.5.  KF_FP64 needs 150 registers, which the staged kernel's 96 spill:
+  // 1,000,000 tracks p2r 663 and 681 us, p2z 463 and 464; 30,000: 40 and 50,
+  // 29 and 35; 2,000: 17 and 30, 12 and 21.
+  LaunchConfig cfg{KF_STEP_DIRECT, kDirectThreads, 2};
   if (plain_loads) {
     // host or managed memory: the grid-stride kernel below
   } else if (const LaunchConfig *o = thread_override()) {
