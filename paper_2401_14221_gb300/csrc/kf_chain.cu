@@ -20,6 +20,7 @@
 #include "kf_device.cuh"
 #include "kf_step.cuh"
 #include "kf_chain.cuh"
+#include "kf_fp64_group.cuh"
 
 namespace kf {
 namespace staged {
@@ -116,12 +117,19 @@ __device__ __forceinline__ void chain_redo_track(const ChainArgs &a, int64_t i) 
   a.status[i] = (uint8_t)st;
 }
 
-// The second pass over one list of the whole batch's marked tracks, 32 to
-// a warp.  An FP64 warp instruction occupies the FP64 pipe as long with one
-// lane active as with 32 (spreading a span's marks over two warps instead
-// of one made the adaptive chain slower, 0.761 -> 0.795 ms), so full warps
-// need about a quarter fewer FP64 warp instructions than one partly filled
-// warp per span; one-warp blocks, four per SM, spread them over the SMs.
+// The same for 32 tracks by the block's four warps (kf_fp64_group.cuh).
+__device__ __forceinline__ void chain_redo_group(const ChainArgs &a, const f64::Group &g,
+                                                 int64_t i, bool store) {
+  const ChainLoc l6 = chain_locate<6>(i, a.n, a.soa, a.lw);
+  const ChainLoc l21 = chain_locate<21>(i, a.n, a.soa, a.lw);
+  const ChainLoc l3 = chain_locate<3>(i, a.n, a.soa, a.lw);
+  const unsigned st =
+      f64::group_chain(g, {a.state, a.cov, a.state, a.cov, l6, l21}, (float)a.charge[i], a.bz, a.L,
+                       a.kinds, a.pos, a.hits, a.hit_stride, a.hitcovs, a.hc_stride, l3, store);
+  if (g.role == 0 && store && a.status) a.status[i] = (uint8_t)st;
+}
+
+// The second pass over one list of the whole batch's marked tracks.
 // chain_compact_kernel builds the list: each block gathers its span's marks
 // and appends them (one atomic per block; the order of the list varies from
 // run to run, the result of each track does not).
@@ -142,26 +150,53 @@ __global__ void __launch_bounds__(kRedoThreads) chain_compact_kernel(const uint8
 }
 
 constexpr int kRedoListBlocksPerSm = 4;
+// Up to this many tracks per SM four warps share 32 tracks, beyond it each
+// thread runs a track.  KF_FP64 chain of 15 layers, us: one group per SM (up
+// to 4,864 tracks) 91, two 122, three 167, four 214; one thread per track 163
+// up to 10,000 tracks, 175 up to 19,000.
+constexpr int kGroupTracksPerSm = 96;
 
-__global__ void __launch_bounds__(32) chain_redo_list_kernel(const ChainArgs a,
-                                                             const uint32_t *count,
-                                                             const uint32_t *list) {
+__global__ void __launch_bounds__(kRedoThreads, kRedoListBlocksPerSm)
+    chain_redo_list_kernel(const ChainArgs a, const uint32_t *count, const uint32_t *list) {
+  __shared__ f64::Shared sh;
   const int64_t total = *count;
-  for (int64_t g = blockIdx.x; g * 32 < total; g += gridDim.x) {
-    const int64_t q = g * 32 + threadIdx.x;
-    if (q < total) chain_redo_track(a, list[q]);
+  if (total > (int64_t)(gridDim.x / kRedoListBlocksPerSm) * kGroupTracksPerSm) {
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
+         q += (int64_t)gridDim.x * blockDim.x)
+      chain_redo_track(a, list[q]);
+    return;
   }
+  const f64::Group g{sh, (int)threadIdx.x >> 5, (int)threadIdx.x & 31};
+  for (int64_t base = (int64_t)blockIdx.x * 32; base < total; base += (int64_t)gridDim.x * 32)
+    chain_redo_group(a, g, list[f64::group_place(base, total, g.lane)], base + g.lane < total);
 }
 
 // KF_ADAPTIVE's second pass without a list (no scratch memory could be had,
 // or more than 2^32 - 1 tracks): each block gathers the marked tracks of its
 // span (gather_marked) and reruns them.
-__global__ void __launch_bounds__(kRedoThreads) chain_redo_kernel(const ChainArgs a) {
+__global__ void __launch_bounds__(kRedoThreads, 4) chain_redo_kernel(const ChainArgs a) {
+  __shared__ f64::Shared sh;
   __shared__ uint16_t list[kRedoSpan];
   __shared__ int count;
   const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
   const int cnt = gather_marked(a.status, span0, a.n, list, &count);
-  for (int q = threadIdx.x; q < cnt; q += blockDim.x) chain_redo_track(a, span0 + list[q]);
+  if (cnt > f64::kGroupMax) {
+    for (int q = threadIdx.x; q < cnt; q += blockDim.x) chain_redo_track(a, span0 + list[q]);
+    return;
+  }
+  const f64::Group g{sh, (int)threadIdx.x >> 5, (int)threadIdx.x & 31};
+  for (int base = 0; base < cnt; base += 32)
+    chain_redo_group(a, g, span0 + list[f64::group_place(base, cnt, g.lane)],
+                     base + g.lane < cnt);
+}
+
+// KF_FP64 for batches too small to give every scheduler a warp of tracks.
+__global__ void __launch_bounds__(kRedoThreads, kRedoListBlocksPerSm)
+    chain_group_kernel(const ChainArgs a) {
+  __shared__ f64::Shared sh;
+  const f64::Group g{sh, (int)threadIdx.x >> 5, (int)threadIdx.x & 31};
+  const int64_t base = (int64_t)blockIdx.x * 32;
+  chain_redo_group(a, g, f64::group_place(base, a.n, g.lane), base + g.lane < a.n);
 }
 
 // A stream-ordered memory pool per device for the second pass's list,
@@ -219,8 +254,8 @@ int launch_chain_redo(const ChainArgs &a, cudaStream_t s) {
       rc = check_cuda(cudaGetLastError(), "chain compaction launch");
     }
     if (rc == KF_OK) {
-      chain_redo_list_kernel<<<(unsigned)(kRedoListBlocksPerSm * sms), 32, 0, s>>>(a, count,
-                                                                                  list);
+      chain_redo_list_kernel<<<(unsigned)(kRedoListBlocksPerSm * sms), kRedoThreads, 0, s>>>(
+          a, count, list);
       rc = check_cuda(cudaGetLastError(), "chain redo pass launch");
     }
     const cudaError_t freed = cudaFreeAsync(buf, s);  // returned to the pool on every path
@@ -305,6 +340,15 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   const int64_t blocks = (d.n + threads - 1) / threads;
   if (blocks > 0x7fffffffLL) return set_error(KF_ERR_ARG, "n too large for one launch");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (params->precision == KF_FP64) {  // few tracks: four warps to 32 of them
+    int dev = 0, sms = 0;
+    if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
+    if (int rc = staged::sm_count(dev, &sms)) return rc;
+    if (d.n <= (int64_t)sms * kGroupTracksPerSm) {
+      chain_group_kernel<<<(unsigned)((d.n + 31) / 32), kRedoThreads, 0, s>>>(a);
+      return check_cuda(cudaGetLastError(), "chain launch");
+    }
+  }
   switch (params->precision) {
     case KF_FP32: chain_kernel<kFP32><<<(unsigned)blocks, threads, 0, s>>>(a); break;
     case KF_FP64_UPDATE: chain_kernel<kFP64Update><<<(unsigned)blocks, threads, 0, s>>>(a); break;

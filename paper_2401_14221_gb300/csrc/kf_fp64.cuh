@@ -13,7 +13,7 @@
 //  * 1/x, 1/sqrt(x) and sqrt(x) from an FP32 seed and one third-order step
 //    (3 to 5 FP64 instructions; the library's take 6 to 9);
 //  * sin and cos from a 256-entry table (13 FP64 instructions, the library's
-//    27), the turning angle from atan2f and one correction (16 instead of 45);
+//    27), the turning angle from the same table (9 instead of 45);
 //  * the transport C' = J C J^T through J's factored form J = J_s + u (ds/dp)
 //    (89 multiply-adds for a cylinder, 70 for a plane), and the update
 //    without the columns and products the general form spends on them.
@@ -206,9 +206,16 @@ constexpr SinCosTable make() {
 
 __device__ constexpr SinCosTable kSinCos = table::make();
 
+constexpr double kStepHi = 0.02454369260617026, kStepLo = 9.567553118338697e-19;  // pi/128
+
 struct sc {
   double s, c;
 };
+
+__device__ __forceinline__ sc table_entry(int k) {
+  const double2 t = __ldg(reinterpret_cast<const double2 *>(&kSinCos.v[k & 255][0]));
+  return {t.x, t.y};
+}
 
 static __device__ __noinline__ sc sincos_any(double x) {
   sc r;
@@ -227,41 +234,50 @@ __device__ __forceinline__ sc sincos(double x) {
   if (top(x) >= 0x40500000u) return sincos_any(x);
   const float kf = rintf(cut(x) * 40.743665431525206f);  // 128 / pi
   const double k = from_float(kf);
-  const double r = fma(k, -9.567553118338697e-19, fma(k, -0.02454369260617026, x));
-  const double2 t =
-      __ldg(reinterpret_cast<const double2 *>(&kSinCos.v[(int)kf & 255][0]));
+  const double r = fma(k, -kStepLo, fma(k, -kStepHi, x));
+  const sc t = table_entry((int)kf);
   const double z = mul(r, r);
   const double sr = fma(mul(r, z), fma(z, 0x1.1110b41d9fc27p-7, -0x1.5555555542e06p-3), r);
   const double cr = mul(z, fma(z, fma(z, -1.0 / 720.0, 1.0 / 24.0), -0.5));
-  return {fma(t.x, cr, fma(t.y, sr, t.x)), fma(t.y, cr, fma(-t.x, sr, t.y))};
+  return {fma(t.s, cr, fma(t.c, sr, t.s)), fma(t.c, cr, fma(-t.s, sr, t.c))};
 }
 
 static __device__ __noinline__ double atan2_any(double y, double x) { return ::atan2(y, x); }
 
 // atan2(y, x) when its sine and cosine are known (y and x over their norm):
-// with the float angle h0, sin(h - h0) = sh cos h0 - ch sin h0 is at most
-// 1e-6 and is the correction (its cube is below 1e-18 of it).
+// atan2f names the nearest table angle k pi/128, s = sin(h - k pi/128) comes
+// from the table's entries, and its arcsine from the series to s^7 (|s| <=
+// 0.0123: the next term is 2e-17 of it).  9 FP64 instructions; the library's
+// atan2 takes 45, a correction of atan2f through sincos 16.
 __device__ __forceinline__ double angle(double y, double x, double sh, double ch) {
   if (top(y) >= 0x46300000u || top(x) >= 0x46300000u) return atan2_any(y, x);  // 2^100, NaN
-  const double h0 = from_float(atan2f(cut(y), cut(x)));
-  const sc a = sincos(h0);
-  return add(h0, fma(sh, a.c, -mul(ch, a.s)));
+  const float kf = rintf(atan2f(cut(y), cut(x)) * 40.743665431525206f);
+  const double k = from_float(kf);
+  const sc t = table_entry((int)kf);
+  const double s = fma(sh, t.c, -mul(ch, t.s)), z = mul(s, s);
+  const double d = fma(mul(s, z), fma(z, fma(z, 15.0 / 336.0, 3.0 / 40.0), 1.0 / 6.0), s);
+  return fma(k, kStepHi, fma(k, kStepLo, d));
 }
 
 // S(h) = sin(h)/h and dS/dh from sin(h) and cos(h); below |h| = 0.05, where
 // cos(h) - S(h) cancels, the Taylor series (the first terms left out are
-// below 1e-18 and 3e-17 of the sums).
-__device__ __forceinline__ void sinc(double h, double sh, double ch, double &S, double &dS) {
-  if (top(h) < 0x3fa99999u) {  // 0.05
-    const double z = mul(h, h);
-    S = fma(z,
-            fma(z, fma(z, fma(z, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0);
-    dS = mul(h, fma(z, fma(z, fma(z, 1.0 / 45360.0, -1.0 / 840.0), 1.0 / 30.0), -1.0 / 3.0));
-  } else {
-    const double ih = rcp(h);
-    S = mul(sh, ih);
-    dS = mul(sub(ch, S), ih);
-  }
+// below 1e-18 and 3e-17 of the sums), else with 1/h.
+struct Sinc {
+  double S, dS;
+};
+__device__ __forceinline__ bool sinc_by_series(double h) { return top(h) < 0x3fa99999u; }
+__device__ __forceinline__ Sinc sinc_series(double h) {
+  const double z = mul(h, h);
+  return {fma(z, fma(z, fma(z, fma(z, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0),
+              1.0),
+          mul(h, fma(z, fma(z, fma(z, 1.0 / 45360.0, -1.0 / 840.0), 1.0 / 30.0), -1.0 / 3.0))};
+}
+__device__ __forceinline__ Sinc sinc_quotient(double ih, double sh, double ch) {
+  const double S = mul(sh, ih);
+  return {S, mul(sub(ch, S), ih)};
+}
+__device__ __forceinline__ Sinc sinc(double h, double sh, double ch) {
+  return sinc_by_series(h) ? sinc_series(h) : sinc_quotient(rcp(h), sh, ch);
 }
 
 // Azimuth wrapped to (-pi, pi] (as wrap_phi, kf_device.cuh).  The number of
@@ -277,56 +293,231 @@ __device__ __forceinline__ double wrap_phi(double a) {
   return w;
 }
 
-// ------------------------------------------------------------------- steps
+// ------------------------------------------------------------------- pieces
+// Each piece of a step is a function of its own, so that the step of one
+// thread (below) and the step that four warps share (kf_fp64_group.cuh)
+// round alike.
 
-// The Kalman update of both step kinds, on the five components that carry
-// variance: index M0 of p and C is the first measured component (with weight
-// h0, 1 on a plane), M1 the second, a, b, c the other three.  C holds C', p
-// the propagated state, r0, r1 the residual.  The measured rows and columns
-// use C'' H^T = K V, which cancels no digits; the rest C' - K (H C').
-// Returns kSNotPD and leaves p and C alone if S is not positive definite.
-template <int M0, int M1, bool UNIT0>
-__device__ __forceinline__ unsigned update(double (&p)[6], double (&C)[21], double h0, double V00,
-                                           double V01, double V11, double r0, double r1) {
-  constexpr int kRest[3] = {3, 4, 5};
-  constexpr int kAll[5] = {M0, M1, 3, 4, 5};
-  const double T0 = C[tri(M0, M0)], T1 = C[tri(M1, M0)], U1 = C[tri(M1, M1)];
+// d omega / d k
+__device__ __forceinline__ double curvature_rate(double q, double bz) {
+  return mul(mul(q, -0.299792458e-2), bz);
+}
+
+// cos and sin of the chord's direction phi + h.
+__device__ __forceinline__ sc turned(const sc &ph, const sc &h) {
+  return {fma(ph.c, h.s, mul(ph.s, h.c)), fma(ph.c, h.c, -mul(ph.s, h.s))};
+}
+
+// The update's gain (two measured components, h0 the first one's weight):
+// K0 = t a00 + u Si01, K1 = t a01 + u Si11 for a component with C' entries t
+// and u in the measured columns.  bad: S is not positive definite.
+struct Gain {
+  double a00, a01, Si01, Si11;
+  bool bad;
+};
+template <bool UNIT0>
+__device__ __forceinline__ Gain gain(double T0, double T1, double U1, double h0, double V00,
+                                     double V01, double V11) {
   const double S00 = UNIT0 ? add(T0, V00) : fma(mul(h0, h0), T0, V00);
   const double S01 = UNIT0 ? add(T1, V01) : fma(h0, T1, V01);
   const double S11 = add(U1, V11);
   const double det = fma(S00, S11, -mul(S01, S01));
-  if (!(gt0(S00) && gt0(det))) return kSNotPD;
+  Gain g;
+  g.bad = !(gt0(S00) && gt0(det));
   const double inv = rcp(det);
-  const double Si00 = mul(S11, inv), Si01 = -mul(S01, inv), Si11 = mul(S00, inv);
-  const double a00 = UNIT0 ? Si00 : mul(h0, Si00), a01 = UNIT0 ? Si01 : mul(h0, Si01);
-  double K0[6], K1[6];
+  const double Si00 = mul(S11, inv);
+  g.Si01 = -mul(S01, inv);
+  g.Si11 = mul(S00, inv);
+  g.a00 = UNIT0 ? Si00 : mul(h0, Si00);
+  g.a01 = UNIT0 ? g.Si01 : mul(h0, g.Si01);
+  return g;
+}
+struct Pair {
+  double a, b;
+};
+__device__ __forceinline__ Pair gain_of(const Gain &g, double t, double u) {
+  return {fma(t, g.a00, mul(u, g.Si01)), fma(t, g.a01, mul(u, g.Si11))};
+}
+// k.a x + k.b y + c, and without c: the state's update, and a measured
+// column, K V.
+__device__ __forceinline__ double dot_add(const Pair &k, double x, double y, double c) {
+  return fma(k.a, x, fma(k.b, y, c));
+}
+__device__ __forceinline__ double dot(const Pair &k, double x, double y) {
+  return fma(k.a, x, mul(k.b, y));
+}
+// C'_im - K_i (H C')_m with k = (h0 K0, K1) of row i, t and u of row m.
+__device__ __forceinline__ double reduced(const Pair &k, double t, double u, double c) {
+  return fma(-k.a, t, fma(-k.b, u, c));
+}
+
+// --------------------------------------------------------------- p2z pieces
+// The path to the plane: s, the half turning angle h, ds/dz, ds/dtheta.
+// Not ok: parallel to the plane.
+struct PlanePath {
+  double s, h, dsz, dst;
+  bool ok;
+};
+__device__ __forceinline__ PlanePath plane_path(const sc &th, double dz, double w) {
+  PlanePath r;
+  r.ok = abs_gt(th.c, 0x3f1a36e2eb1c432dull);  // 1e-4
+  const double ict = rcp(th.c), tanth = mul(th.s, ict);
+  r.s = mul(dz, tanth);
+  r.h = mul(mul(0.5, w), r.s);
+  r.dsz = -tanth;
+  r.dst = mul(mul(dz, ict), ict);
+  return r;
+}
+
+// Chord L and the factors of the partials along k at fixed path: with the
+// chord's direction (c, s), d(x, y)/dk = a (c, s) + b (-s, c); kap = d phi/dk,
+// hs2 = s kap / 2.
+struct Bend {
+  double L, a, b;
+};
+__device__ __forceinline__ double half_s_kap(double s, double kap) {
+  return mul(mul(0.5, s), kap);
+}
+__device__ __forceinline__ Bend bend(double s, double hs2, const Sinc &c) {
+  return {mul(s, c.S), mul(hs2, c.dS), mul(hs2, c.S)};
+}
+
+// A row e_i + a e_k + b e_phi of J_s times a column (c_i, c_k, c_phi) of C.
+__device__ __forceinline__ double row(double a, double b, double ci, double ck, double cf) {
+  return fma(b, cf, fma(a, ck, ci));
+}
+
+// --------------------------------------------------------------- p2r pieces
+// The crossing (cos h, sin h, chord) = (den, yh, d) / hypot(den, yh), as in
+// propagate_to_r (kf_device.cuh) with half the curvature wh = omega/2 and
+// yh = wh d.  Not ok: starts outside, or never reaches the cylinder (the rest
+// is then a crossing on the spot, which four warps carry through the step to
+// no effect and without a division by zero).
+struct Cross {
+  double d, den, yh, ch, sh, L;
+  bool ok;
+};
+__device__ __forceinline__ Cross cross(double x, double y, const sc &ph, double w, double wh,
+                                       double R) {
+  Cross r{};
+  r.d = fma(R, R, -fma(x, x, mul(y, y)));
+  const double A = fma(x, ph.c, mul(y, ph.s)), B = fma(y, ph.c, -mul(x, ph.s));
+  r.yh = mul(wh, r.d);
+  const double D = fma(A, A, mul(fma(w, B, fma(-wh, r.yh, 1.0)), r.d));
+  r.ok = gt0(r.d) && ge0(D);
+  if (!r.ok) {
+    r.den = r.ch = 1.0;
+    return r;
+  }
+  r.den = add(A, sqrt(D));
+  const double inv = rsqrt(fma(r.den, r.den, mul(r.yh, r.yh)));
+  r.ch = mul(r.den, inv);
+  r.sh = mul(r.yh, inv);
+  r.L = mul(r.d, inv);
+  return r;
+}
+
+// The path for the half turning angle h: 2 h / omega (iwh = 2 / omega), or the
+// straight line's.
+__device__ __forceinline__ double arc(const Cross &c, double h, double w, double iwh) {
+  return top(w) > 0x3d719799u ? mul(h, iwh) : mul(c.d, rcp(c.den));  // 1e-12
+}
+
+// Surface frame at the crossing, n = (ca, sa), t = (-sa, ca), with the chord's
+// direction (nm, tm) in it; the gradient of the path is ds = -ic m with
+// m = n.J_s = (ca, sa, ., mk, mf, .).
+struct Frame {
+  double x, y, ca, sa, nm, tm, mf;
+};
+__device__ __forceinline__ Frame frame(const sc &e, double L, double x, double y, double iR) {
+  Frame r;
+  r.x = fma(L, e.c, x);
+  r.y = fma(L, e.s, y);
+  r.ca = mul(r.x, iR);
+  r.sa = mul(r.y, iR);
+  r.nm = fma(r.ca, e.c, mul(r.sa, e.s));
+  r.tm = fma(r.ca, e.s, -mul(r.sa, e.c));
+  r.mf = -mul(L, r.tm);
+  return r;
+}
+// The track's direction (nu, tu) in the frame, the chord's turned by h; ic =
+// 1 / nu, tau = tu / nu and the t row v = t.J_s - tau m but for its entry vk.
+struct Slope {
+  double ic, tau, vx, vy, vf;
+};
+__device__ __forceinline__ Slope slope(const Frame &f, double ch, double sh, double L) {
+  Slope r;
+  const double nu = fma(f.nm, ch, -mul(f.tm, sh)), tu = fma(f.tm, ch, mul(f.nm, sh));
+  r.ic = rcp(nu);
+  r.tau = mul(tu, r.ic);
+  r.vx = fma(-r.tau, f.ca, -f.sa);
+  r.vy = fma(-r.tau, f.sa, f.ca);
+  r.vf = fma(-r.tau, f.mf, mul(L, f.nm));
+  return r;
+}
+// (mk, vk): the entries of m and v along k.
+__device__ __forceinline__ Pair along_k(double a, double b, double nm, double tm, double tau) {
+  const double mk = fma(a, nm, -mul(b, tm));
+  return {mk, fma(-tau, mk, fma(a, tm, mul(b, nm)))};
+}
+// A row (m0, m1, mk, mf) over (x, y, k, phi) times a column: the part without
+// k (known before the turning angle is), and the whole.
+__device__ __forceinline__ double part(double m0, double m1, double mf, double c0, double c1,
+                                       double c4) {
+  return fma(mf, c4, fma(m1, c1, mul(m0, c0)));
+}
+
+// Measurement direction at the hit, u = (-hy, hx) / |h|, and V = P V_hit P^T.
+struct HitFrame {
+  double ux, uy, V00, V01;
+};
+__device__ __forceinline__ HitFrame hit_frame(double hx, double hy, const double (&hc)[6]) {
+  HitFrame r;
+  const double ir = rsqrt(fma(hx, hx, mul(hy, hy)));
+  r.ux = -mul(hy, ir);
+  r.uy = mul(hx, ir);
+  r.V00 = fma(r.ux, fma(r.ux, hc[0], mul(r.uy, hc[1])),
+              mul(r.uy, fma(r.ux, hc[1], mul(r.uy, hc[2]))));
+  r.V01 = fma(r.ux, hc[3], mul(r.uy, hc[4]));
+  return r;
+}
+
+// ------------------------------------------------------------------- steps
+
+// The Kalman update of both step kinds, on the five components that carry
+// variance: index M0 of p and C is the first measured component (with weight
+// h0, 1 on a plane), M1 the second, 3, 4, 5 the others.  C holds C', p the
+// propagated state, r0, r1 the residual.  The measured rows and columns use
+// C'' H^T = K V, which cancels no digits; the rest C' - K (H C').  Returns
+// kSNotPD and leaves p and C alone if S is not positive definite.
+template <int M0, int M1, bool UNIT0>
+__device__ __forceinline__ unsigned update(double (&p)[6], double (&C)[21], double h0, double V00,
+                                           double V01, double V11, double r0, double r1) {
+  constexpr int kAll[5] = {M0, M1, 3, 4, 5};
+  const Gain g = gain<UNIT0>(C[tri(M0, M0)], C[tri(M1, M0)], C[tri(M1, M1)], h0, V00, V01, V11);
+  if (g.bad) return kSNotPD;
+  Pair K[6];
 #pragma unroll
   for (int e = 0; e < 5; ++e) {
     const int i = kAll[e];
-    const double t = C[tri(i, M0)], u = C[tri(i, M1)];
-    K0[i] = fma(t, a00, mul(u, Si01));
-    K1[i] = fma(t, a01, mul(u, Si11));
-    p[i] = fma(K0[i], r0, fma(K1[i], r1, p[i]));
+    K[i] = gain_of(g, C[tri(i, M0)], C[tri(i, M1)]);
+    p[i] = dot_add(K[i], r0, r1, p[i]);
   }
   // the unmeasured block first: it needs C's measured columns as they were
 #pragma unroll
-  for (int e = 0; e < 3; ++e) {
-    const int i = kRest[e];
-    const double k0 = UNIT0 ? K0[i] : mul(h0, K0[i]);
+  for (int i = 3; i < 6; ++i) {
+    const Pair k{UNIT0 ? K[i].a : mul(h0, K[i].a), K[i].b};
 #pragma unroll
-    for (int f = 0; f <= e; ++f) {
-      const int m = kRest[f];
-      C[tri(i, m)] =
-          fma(-k0, C[tri(m, M0)], fma(-K1[i], C[tri(m, M1)], C[tri(i, m)]));
-    }
+    for (int m = 3; m <= i; ++m)
+      C[tri(i, m)] = reduced(k, C[tri(m, M0)], C[tri(m, M1)], C[tri(i, m)]);
   }
   const double ih = UNIT0 ? 1.0 : rcp(h0);
   const double W00 = UNIT0 ? V00 : mul(V00, ih), W01 = UNIT0 ? V01 : mul(V01, ih);
 #pragma unroll
   for (int e = 0; e < 5; ++e) {
     const int i = kAll[e];
-    C[tri(i, M0)] = fma(K0[i], W00, mul(K1[i], W01));
-    if (i != M0) C[tri(i, M1)] = fma(K0[i], V01, mul(K1[i], V11));
+    C[tri(i, M0)] = dot(K[i], W00, W01);
+    if (i != M0) C[tri(i, M1)] = dot(K[i], V01, V11);
   }
   return 0u;
 }
@@ -342,58 +533,42 @@ __device__ __forceinline__ unsigned update(double (&p)[6], double (&C)[21], doub
 __device__ __forceinline__ unsigned p2z_step(double (&p)[6], double (&C)[21], double q, double bz,
                                              double zt, double hx, double hy, double vxx,
                                              double vxy, double vyy) {
-  const sc th = sincos(p[5]);
-  if (!abs_gt(th.c, 0x3f1a36e2eb1c432dull)) return kNoIntersect;  // 1e-4
-  const sc ph = sincos(p[4]);
-  const double ict = rcp(th.c);
-  const double tanth = mul(th.s, ict);
-  const double dz = sub(zt, p[2]);
-  const double s = mul(dz, tanth);
-  const double dw = mul(mul(q, -0.299792458e-2), bz);
-  const double w = mul(dw, p[3]);
-  const double h = mul(mul(0.5, w), s);
-  const sc hh = sincos(h);
-  double S, dS;
-  sinc(h, hh.s, hh.c, S, dS);
-  const double L = mul(s, S);
-  const double cm = fma(ph.c, hh.c, -mul(ph.s, hh.s)), sm = fma(ph.c, hh.s, mul(ph.s, hh.c));
-  const double c1 = fma(cm, hh.c, -mul(sm, hh.s)), s1 = fma(cm, hh.s, mul(sm, hh.c));
-  const double kap = mul(s, dw);
-  const double hs2 = mul(mul(0.5, s), kap);
-  const double a = mul(hs2, dS), b = mul(hs2, S);
-  const double Xk = fma(a, cm, -mul(b, sm)), Yk = fma(a, sm, mul(b, cm));
-  const double Xf = -mul(L, sm), Yf = mul(L, cm);
-  const double dsz = -tanth, dst = mul(mul(dz, ict), ict);
-  p[0] = fma(L, cm, p[0]);
-  p[1] = fma(L, sm, p[1]);
+  const double dw = curvature_rate(q, bz), w = mul(dw, p[3]);
+  const PlanePath pa = plane_path(sincos(p[5]), sub(zt, p[2]), w);
+  if (!pa.ok) return kNoIntersect;
+  const sc hh = sincos(pa.h);
+  const double kap = mul(pa.s, dw);
+  const Bend be = bend(pa.s, half_s_kap(pa.s, kap), sinc(pa.h, hh.s, hh.c));
+  const sc e = turned(sincos(p[4]), hh), f = turned(e, hh);
+  const double Xk = fma(be.a, e.c, -mul(be.b, e.s)), Yk = fma(be.a, e.s, mul(be.b, e.c));
+  const double Xf = -mul(be.L, e.s), Yf = mul(be.L, e.c);
+  p[0] = fma(be.L, e.c, p[0]);
+  p[1] = fma(be.L, e.s, p[1]);
   p[2] = zt;
-  p[4] = fma(2.0, h, p[4]);
+  p[4] = fma(2.0, pa.h, p[4]);
 
-  const double *Z[6] = {&C[3], &C[4], &C[5], &C[8], &C[12], &C[17]};      // row z of C
-  const double *T[6] = {&C[15], &C[16], &C[17], &C[18], &C[19], &C[20]};  // row theta
   double c[6];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) c[j] = fma(dsz, *Z[j], mul(dst, *T[j]));
-  const double dd = fma(dsz, c[2], mul(dst, c[5]));
-  const double ex = fma(Xf, c[4], fma(Xk, c[3], c[0]));
-  const double ey = fma(Yf, c[4], fma(Yk, c[3], c[1]));
+  for (int j = 0; j < 6; ++j) c[j] = fma(pa.dsz, C[tri(2, j)], mul(pa.dst, C[tri(5, j)]));
+  const double dd = fma(pa.dsz, c[2], mul(pa.dst, c[5]));
+  const double ex = row(Xk, Xf, c[0], c[3], c[4]), ey = row(Yk, Yf, c[1], c[3], c[4]);
   const double ef = fma(kap, c[3], c[4]);
-  const double gx = fma(c1, dd, ex), gy = fma(s1, dd, ey), gf = fma(w, dd, ef);
-  auto X = [&](int j) { return fma(Xf, C[tri(4, j)], fma(Xk, C[tri(3, j)], C[tri(0, j)])); };
-  auto Y = [&](int j) { return fma(Yf, C[tri(4, j)], fma(Yk, C[tri(3, j)], C[tri(1, j)])); };
+  const double gx = fma(f.c, dd, ex), gy = fma(f.s, dd, ey), gf = fma(w, dd, ef);
+  auto X = [&](int j) { return row(Xk, Xf, C[tri(0, j)], C[tri(3, j)], C[tri(4, j)]); };
+  auto Y = [&](int j) { return row(Yk, Yf, C[tri(1, j)], C[tri(3, j)], C[tri(4, j)]); };
   auto F = [&](int j) { return fma(kap, C[tri(3, j)], C[tri(4, j)]); };
   const double xk = X(3), xf = X(4), yk = Y(3), yf = Y(4), fk = F(3), ff = F(4);
-  const double xx = fma(Xf, xf, fma(Xk, xk, X(0))), xy = fma(Yf, xf, fma(Yk, xk, X(1)));
-  const double yy = fma(Yf, yf, fma(Yk, yk, Y(1)));
-  const double xt = fma(c1, c[5], X(5)), yt = fma(s1, c[5], Y(5)), ft = fma(w, c[5], F(5));
-  C[tri(0, 0)] = fma(c1, gx, fma(c1, ex, xx));
-  C[tri(1, 0)] = fma(c1, gy, fma(s1, ex, xy));
-  C[tri(1, 1)] = fma(s1, gy, fma(s1, ey, yy));
-  C[tri(4, 0)] = fma(c1, gf, fma(w, ex, fma(kap, xk, xf)));
-  C[tri(4, 1)] = fma(s1, gf, fma(w, ey, fma(kap, yk, yf)));
+  const double xx = row(Xk, Xf, X(0), xk, xf), xy = row(Yk, Yf, X(1), xk, xf);
+  const double yy = row(Yk, Yf, Y(1), yk, yf);
+  const double xt = fma(f.c, c[5], X(5)), yt = fma(f.s, c[5], Y(5)), ft = fma(w, c[5], F(5));
+  C[tri(0, 0)] = fma(f.c, gx, fma(f.c, ex, xx));
+  C[tri(1, 0)] = fma(f.c, gy, fma(f.s, ex, xy));
+  C[tri(1, 1)] = fma(f.s, gy, fma(f.s, ey, yy));
+  C[tri(4, 0)] = fma(f.c, gf, fma(w, ex, fma(kap, xk, xf)));
+  C[tri(4, 1)] = fma(f.s, gf, fma(w, ey, fma(kap, yk, yf)));
   C[tri(4, 4)] = fma(w, gf, fma(w, ef, fma(kap, fk, ff)));
-  C[tri(3, 0)] = fma(c1, c[3], xk);
-  C[tri(3, 1)] = fma(s1, c[3], yk);
+  C[tri(3, 0)] = fma(f.c, c[3], xk);
+  C[tri(3, 1)] = fma(f.s, c[3], yk);
   C[tri(4, 3)] = fma(w, c[3], fk);
   C[tri(5, 0)] = xt;
   C[tri(5, 1)] = yt;
@@ -411,114 +586,82 @@ __device__ __forceinline__ unsigned p2z_step(double (&p)[6], double (&C)[21], do
 // with the hit's azimuth and z.  p and C are left alone when the track starts
 // outside the cylinder or does not reach it.
 //
-// The crossing as in propagate_to_r (kf_device.cuh), with half the curvature
-// wh = omega/2 and yh = wh d, so that (cos h, sin h, chord) = (den, yh, d) /
-// hypot(den, yh).  In the surface frame n = (ca, sa), t = (-sa, ca) the path
-// derivative is ds = -m/(n.u) with m = n.J_s = (ca, sa, ., mk, mf, .), so J's
-// rows are
-//   t: v = t.J_s - tau m (tau = (t.u)/(n.u)),  z: e_z + zt e_theta + cz m,
-//   phi: e_phi + kap e_k + cf m,
-// and C' needs only the two products C m^T and C v^T.  The directions come
-// from rotating (n.e, t.e), e the chord's direction, by the half angle.
+// In the surface frame (Axes) J's rows are t: v, z: e_z + zt e_theta + cz m,
+// phi: e_phi + kap e_k + cf m, so C' needs only the two products C m^T and
+// C v^T.
 __device__ __forceinline__ unsigned p2r_step(double (&p)[6], double (&C)[21], double q, double bz,
                                              double R, double hx, double hy, double hz,
                                              const double (&hc)[6]) {
-  const double x = p[0], y = p[1];
-  const double d = fma(R, R, -fma(x, x, mul(y, y)));
-  if (!gt0(d)) return kNoIntersect;
+  const double dw = curvature_rate(q, bz), w = mul(dw, p[3]), wh = mul(0.5, w);
   const sc ph = sincos(p[4]);
-  const double dw = mul(mul(q, -0.299792458e-2), bz);
-  const double w = mul(dw, p[3]), wh = mul(0.5, w);
-  const double A = fma(x, ph.c, mul(y, ph.s)), B = fma(y, ph.c, -mul(x, ph.s));
-  const double yh = mul(wh, d);
-  const double D = fma(A, A, mul(fma(w, B, fma(-wh, yh, 1.0)), d));
-  if (!ge0(D)) return kNoIntersect;
+  const Cross cr = cross(p[0], p[1], ph, w, wh, R);
+  if (!cr.ok) return kNoIntersect;
   const sc th = sincos(p[5]);
-  const double den = add(A, sqrt(D));
-  const double inv = rsqrt(fma(den, den, mul(yh, yh)));
-  const double ch = mul(den, inv), sh = mul(yh, inv), L = mul(d, inv);
-  const double h = angle(yh, den, sh, ch);
-  const double s =
-      top(w) > 0x3d719799u ? mul(h, rcp(wh)) : mul(d, rcp(den));  // 1e-12; 2 h / omega
-  double S, dS;
-  sinc(h, sh, ch, S, dS);
-  const double cm = fma(ph.c, ch, -mul(ph.s, sh)), sm = fma(ph.c, sh, mul(ph.s, ch));
   const double ist = rcp(th.s), cot = mul(th.c, ist);
-  p[0] = fma(L, cm, x);
-  p[1] = fma(L, sm, y);
+  const double h = angle(cr.yh, cr.den, cr.sh, cr.ch), s = arc(cr, h, w, rcp(wh));
+  const double kap = mul(s, dw);
+  const Bend be = bend(s, half_s_kap(s, kap), sinc(h, cr.sh, cr.ch));
+  const Frame ax = frame(turned(ph, {cr.sh, cr.ch}), cr.L, p[0], p[1], rcp(R));
+  const Slope sl = slope(ax, cr.ch, cr.sh, cr.L);
+  p[0] = ax.x;
+  p[1] = ax.y;
   p[2] = fma(s, cot, p[2]);
   p[4] = fma(2.0, h, p[4]);
 
-  const double iR = rcp(R);
-  const double ca = mul(p[0], iR), sa = mul(p[1], iR);
-  const double nm = fma(ca, cm, mul(sa, sm)), tm = fma(ca, sm, -mul(sa, cm));
-  const double nu = fma(nm, ch, -mul(tm, sh)), tu = fma(tm, ch, mul(nm, sh));
-  const double kap = mul(s, dw);
-  const double hs2 = mul(mul(0.5, s), kap);
-  const double a = mul(hs2, dS), b = mul(hs2, S);
-  const double ic = rcp(nu), tau = mul(tu, ic);
-  const double cz = -mul(cot, ic), cf = -mul(w, ic);
-  const double zt = -mul(mul(s, ist), ist);
-  // m and v over the components x, y, k, phi
-  const double m[4] = {ca, sa, fma(a, nm, -mul(b, tm)), -mul(L, tm)};
-  const double v[4] = {fma(-tau, ca, -sa), fma(-tau, sa, ca),
-                       fma(-tau, m[2], fma(a, tm, mul(b, nm))), fma(-tau, m[3], mul(L, nm))};
-  double cm_[6], cv[6];  // C m^T, C v^T
+  const Pair ak = along_k(be.a, be.b, ax.nm, ax.tm, sl.tau);
+  const double mk = ak.a, vk = ak.b;
+  const double cz = -mul(cot, sl.ic), cf = -mul(w, sl.ic), zt = -mul(mul(s, ist), ist);
+  double cm[6], cv[6];  // C m^T, C v^T
 #pragma unroll
   for (int j = 0; j < 6; ++j) {
     const double c0 = C[tri(0, j)], c1 = C[tri(1, j)], c3 = C[tri(3, j)], c4 = C[tri(4, j)];
-    cm_[j] = fma(m[3], c4, fma(m[2], c3, fma(m[1], c1, mul(m[0], c0))));
-    cv[j] = fma(v[3], c4, fma(v[2], c3, fma(v[1], c1, mul(v[0], c0))));
+    cm[j] = fma(mk, c3, part(ax.ca, ax.sa, ax.mf, c0, c1, c4));
+    cv[j] = fma(vk, c3, part(sl.vx, sl.vy, sl.vf, c0, c1, c4));
   }
-  const double mm = fma(m[3], cm_[4], fma(m[2], cm_[3], fma(m[1], cm_[1], mul(m[0], cm_[0]))));
-  const double mv = fma(m[3], cv[4], fma(m[2], cv[3], fma(m[1], cv[1], mul(m[0], cv[0]))));
-  const double vv = fma(v[3], cv[4], fma(v[2], cv[3], fma(v[1], cv[1], mul(v[0], cv[0]))));
+  const double mm = fma(mk, cm[3], part(ax.ca, ax.sa, ax.mf, cm[0], cm[1], cm[4]));
+  const double mv = fma(mk, cv[3], part(ax.ca, ax.sa, ax.mf, cv[0], cv[1], cv[4]));
+  const double vv = fma(vk, cv[3], part(sl.vx, sl.vy, sl.vf, cv[0], cv[1], cv[4]));
   const double Czk = C[tri(3, 2)], Czf = C[tri(4, 2)], Czt = C[tri(5, 2)];
   const double Ckk = C[tri(3, 3)], Ckf = C[tri(4, 3)], Ckt = C[tri(5, 3)];
-  const double e1 = fma(zt, cm_[5], cm_[2]), f1 = fma(cz, mm, e1);
-  const double e2 = fma(kap, cm_[3], cm_[4]), f2 = fma(cf, mm, e2);
-  const double gz = fma(zt, C[tri(5, 5)], Czt);           // (C' without the path terms) z, theta
-  const double gf = fma(kap, Ckk, Ckf);                   // phi, k
-  const double gt = fma(kap, Ckt, C[tri(5, 4)]);          // phi, theta
+  const double e1 = fma(zt, cm[5], cm[2]), f1 = fma(cz, mm, e1);
+  const double e2 = fma(kap, cm[3], cm[4]), f2 = fma(cf, mm, e2);
+  const double gz = fma(zt, C[tri(5, 5)], Czt);   // (C' without the path terms) z, theta
+  const double gf = fma(kap, Ckk, Ckf);           // phi, k
+  const double gt = fma(kap, Ckt, C[tri(5, 4)]);  // phi, theta
   C[tri(0, 0)] = vv;
   C[tri(2, 0)] = fma(cz, mv, fma(zt, cv[5], cv[2]));
   C[tri(3, 0)] = cv[3];
   C[tri(4, 0)] = fma(cf, mv, fma(kap, cv[3], cv[4]));
   C[tri(5, 0)] = cv[5];
   C[tri(2, 2)] = fma(cz, add(f1, e1), fma(zt, add(Czt, gz), C[tri(2, 2)]));
-  C[tri(3, 2)] = fma(cz, cm_[3], fma(zt, Ckt, Czk));
+  C[tri(3, 2)] = fma(cz, cm[3], fma(zt, Ckt, Czk));
   C[tri(4, 2)] = fma(cz, f2, fma(cf, e1, fma(zt, gt, fma(kap, Czk, Czf))));
-  C[tri(5, 2)] = fma(cz, cm_[5], gz);
-  C[tri(4, 3)] = fma(cf, cm_[3], gf);
+  C[tri(5, 2)] = fma(cz, cm[5], gz);
+  C[tri(4, 3)] = fma(cf, cm[3], gf);
   C[tri(4, 4)] = fma(cf, add(f2, e2), fma(kap, add(Ckf, gf), C[tri(4, 4)]));
-  C[tri(5, 4)] = fma(cf, cm_[5], gt);
+  C[tri(5, 4)] = fma(cf, cm[5], gt);
 
-  // measurement direction at the hit u = (-hy, hx) / |h|, weight u.t on t
-  const double ir = rsqrt(fma(hx, hx, mul(hy, hy)));
-  const double ux = -mul(hy, ir), uy = mul(hx, ir);
-  const double ut = fma(ca, uy, -mul(sa, ux));
-  const double V00 = fma(ux, fma(ux, hc[0], mul(uy, hc[1])),
-                         mul(uy, fma(ux, hc[1], mul(uy, hc[2]))));
-  const double V01 = fma(ux, hc[3], mul(uy, hc[4]));
-  const double r0 = fma(ux, sub(hx, p[0]), mul(uy, sub(hy, p[1])));
+  const HitFrame hf = hit_frame(hx, hy, hc);
+  const double ut = fma(ax.ca, hf.uy, -mul(ax.sa, hf.ux));  // weight of u on t
+  const double r0 = fma(hf.ux, sub(hx, p[0]), mul(hf.uy, sub(hy, p[1])));
   // the state's t and r offsets start at 0 on the crossing point
   double f[6] = {0.0, 0.0, p[2], p[3], p[4], p[5]};
-  unsigned st = update<0, 2, false>(f, C, ut, V00, V01, hc[5], r0, sub(hz, p[2]));
-  p[0] = fma(-sa, f[0], p[0]);
-  p[1] = fma(ca, f[0], p[1]);
+  unsigned st = update<0, 2, false>(f, C, ut, hf.V00, hf.V01, hc[5], r0, sub(hz, p[2]));
+  p[0] = fma(-ax.sa, f[0], p[0]);
+  p[1] = fma(ax.ca, f[0], p[1]);
 #pragma unroll
   for (int i = 2; i < 6; ++i) p[i] = f[i];
   p[4] = wrap_phi(p[4]);
   // back to (x, y): only the t row and column carry position variance
-  const double tx = -mul(sa, C[tri(0, 0)]), ty = mul(ca, C[tri(0, 0)]);
-  C[tri(0, 0)] = -mul(sa, tx);
-  C[tri(1, 0)] = mul(ca, tx);
-  C[tri(1, 1)] = mul(ca, ty);
+  const double tx = -mul(ax.sa, C[tri(0, 0)]), ty = mul(ax.ca, C[tri(0, 0)]);
+  C[tri(0, 0)] = -mul(ax.sa, tx);
+  C[tri(1, 0)] = mul(ax.ca, tx);
+  C[tri(1, 1)] = mul(ax.ca, ty);
 #pragma unroll
   for (int j = 2; j < 6; ++j) {
     const double t = C[tri(j, 0)];
-    C[tri(j, 0)] = -mul(sa, t);
-    C[tri(j, 1)] = mul(ca, t);
+    C[tri(j, 0)] = -mul(ax.sa, t);
+    C[tri(j, 1)] = mul(ax.ca, t);
   }
   if (!gt0(p[3])) st |= kBadK;
   return st;

@@ -46,6 +46,7 @@
 #include "kf_chain.cuh"
 #include "kf_common.cuh"
 #include "kf_device.cuh"
+#include "kf_fp64_group.cuh"
 #include "kf_host.cuh"
 #include "kf_step.cuh"
 
@@ -136,12 +137,13 @@ __global__ void __launch_bounds__(256) batch_chain_kernel(const __grid_constant_
 }
 
 // KF_ADAPTIVE's second pass over a batch.  Block r covers batch-grid blocks
-// [64 r, 64 r + 64) (4,096 track slots, possibly of several events); it
-// gathers the slots whose track is marked kRedo into shared memory, then its
-// threads rerun those tracks' whole chain in double (chain_track_fp64), so
-// that warps run full.  Every event has a status array (the caller's, for a
-// direct event that gave one, else the arena's).
-constexpr int kBatchRedoBlocks = 64;
+// [16 r, 16 r + 16) (1,024 track slots, possibly of several events); it
+// gathers the slots whose track is marked kRedo into shared memory, then
+// reruns those tracks' whole chain in double as the single chain's second pass
+// does (four warps share 32 tracks, or a thread runs a track where there are
+// more than f64::kGroupMax).  Every event has a status array (the caller's, for
+// a direct event that gave one, else the arena's).
+constexpr int kBatchRedoBlocks = 16;
 
 __device__ __forceinline__ int batch_event_of(const BatchArgs &a, int64_t b) {
   int lo = 0, hi = a.nev - 1;
@@ -153,41 +155,68 @@ __device__ __forceinline__ int batch_event_of(const BatchArgs &a, int64_t b) {
   return lo;
 }
 
-__global__ void __launch_bounds__(256) batch_redo_kernel(const __grid_constant__ BatchArgs a,
-                                                         int64_t nblocks) {
-  __shared__ int16_t ev_of[kBatchRedoBlocks * kBatchThreads];
-  __shared__ int32_t idx_of[kBatchRedoBlocks * kBatchThreads];
+__global__ void __launch_bounds__(kRedoThreads, 4)
+    batch_redo_kernel(const __grid_constant__ BatchArgs a, int64_t nblocks) {
+  constexpr int kSlots = kBatchRedoBlocks * kBatchThreads;
+  constexpr int kAtOnce = 8;  // status bytes a thread has in flight
+  static_assert(kSlots % (kAtOnce * kRedoThreads) == 0 && kSlots <= 65536, "16-bit slots");
+  __shared__ f64::Shared sh;
+  __shared__ uint16_t slot_of[kSlots];
   __shared__ int count;
   if (threadIdx.x == 0) count = 0;
   __syncthreads();
-  for (int slot = threadIdx.x; slot < kBatchRedoBlocks * kBatchThreads; slot += blockDim.x) {
+  // the event and the track of a slot
+  auto event_of = [&](int slot, int64_t &i) -> const EventDesc & {
     const int64_t b = (int64_t)blockIdx.x * kBatchRedoBlocks + slot / kBatchThreads;
-    if (b >= nblocks) break;
-    const int ev = batch_event_of(a, b);
-    const EventDesc &e = a.ev[ev];
-    const int64_t i = (b - e.block_begin) * kBatchThreads + slot % kBatchThreads;
-    if (i < e.n && (e.status[i] & kRedo)) {
-      const int q = atomicAdd(&count, 1);
-      ev_of[q] = (int16_t)ev;
-      idx_of[q] = (int32_t)i;
+    const EventDesc &e = a.ev[batch_event_of(a, b)];
+    i = (b - e.block_begin) * kBatchThreads + slot % kBatchThreads;
+    return e;
+  };
+  for (int s0 = threadIdx.x; s0 < kSlots; s0 += kAtOnce * kRedoThreads) {
+    uint8_t st[kAtOnce];
+#pragma unroll
+    for (int r = 0; r < kAtOnce; ++r) {
+      const int slot = s0 + r * kRedoThreads;
+      st[r] = 0;
+      if ((int64_t)blockIdx.x * kBatchRedoBlocks + slot / kBatchThreads < nblocks) {
+        int64_t i;
+        const EventDesc &e = event_of(slot, i);
+        if (i < e.n) st[r] = e.status[i];
+      }
     }
+#pragma unroll
+    for (int r = 0; r < kAtOnce; ++r)
+      if (st[r] & kRedo) slot_of[atomicAdd(&count, 1)] = (uint16_t)(s0 + r * kRedoThreads);
   }
   __syncthreads();
   const int cnt = count;
-  for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
-    const EventDesc &e = a.ev[ev_of[q]];
-    const int64_t i = idx_of[q];
-    const ChainLoc l6{i, e.n}, l21{i, e.n}, l3{i, e.n};
-    float p[6], C[21];
-    for (int c = 0; c < 6; ++c) p[c] = e.state_in[l6.base + c * l6.stride];
-    for (int k = 0; k < 21; ++k) C[k] = e.cov_in[l21.base + k * l21.stride];
-    const float qf = (float)e.charge[i];
-    unsigned st = chain_track_fp64(p, C, qf, a.bz, a.L, a.kinds, a.pos, e.hits, 3 * e.n,
-                                   e.hitcovs, 6 * e.n, l3, l6);
-    st |= finite_status(p, C);
-    for (int c = 0; c < 6; ++c) e.state_out[l6.base + c * l6.stride] = p[c];
-    for (int k = 0; k < 21; ++k) e.cov_out[l21.base + k * l21.stride] = C[k];
-    e.status[i] = (uint8_t)st;
+  if (cnt > f64::kGroupMax) {
+    for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
+      int64_t i;
+      const EventDesc &e = event_of(slot_of[q], i);
+      const ChainLoc l{i, e.n};
+      float p[6], C[21];
+      for (int c = 0; c < 6; ++c) p[c] = e.state_in[l.base + c * l.stride];
+      for (int k = 0; k < 21; ++k) C[k] = e.cov_in[l.base + k * l.stride];
+      unsigned st = chain_track_fp64(p, C, (float)e.charge[i], a.bz, a.L, a.kinds, a.pos, e.hits,
+                                     3 * e.n, e.hitcovs, 6 * e.n, l, l);
+      st |= finite_status(p, C);
+      for (int c = 0; c < 6; ++c) e.state_out[l.base + c * l.stride] = p[c];
+      for (int k = 0; k < 21; ++k) e.cov_out[l.base + k * l.stride] = C[k];
+      e.status[i] = (uint8_t)st;
+    }
+    return;
+  }
+  const f64::Group g{sh, (int)threadIdx.x >> 5, (int)threadIdx.x & 31};
+  for (int base = 0; base < cnt; base += 32) {
+    int64_t i;
+    const EventDesc &e = event_of(slot_of[f64::group_place(base, cnt, g.lane)], i);
+    const ChainLoc l{i, e.n};
+    const bool mine = base + g.lane < cnt;
+    const unsigned st = f64::group_chain(
+        g, {e.state_in, e.cov_in, e.state_out, e.cov_out, l, l}, (float)e.charge[i], a.bz, a.L,
+        a.kinds, a.pos, e.hits, 3 * e.n, e.hitcovs, 6 * e.n, l, mine);
+    if (g.role == 0 && mine) e.status[i] = (uint8_t)st;
   }
 }
 
@@ -428,7 +457,8 @@ bool launch_batch(kf_server *s, std::vector<Request *> &batch) {
         batch_chain_kernel<kAdaptive><<<g, kBatchThreads, 0, s->s_compute>>>(a);
         e = cudaGetLastError();
         if (e == cudaSuccess)
-          batch_redo_kernel<<<(g + kBatchRedoBlocks - 1) / kBatchRedoBlocks, 256, 0, s->s_compute>>>(
+          batch_redo_kernel<<<(g + kBatchRedoBlocks - 1) / kBatchRedoBlocks, kRedoThreads, 0,
+                              s->s_compute>>>(
               a, (int64_t)g);
         break;
     }

@@ -177,11 +177,40 @@ __global__ void __launch_bounds__(256) step_kernel_strided(const __grid_constant
     step_track<KIND, VARIANT>(a, i);
 }
 
+// The kAdaptive redo of track i of a step launch: read its inputs from
+// global memory, run the step in double, write its outputs and status there.
+// In place is safe: the FP32 kernel did not store this track's result.
+template <int KIND>
+__device__ __forceinline__ void redo_track_fp64(const StepArgs &a, int64_t i) {
+  const Loc l6 = locate<6>(i, a.n, a.soa, a.lw);
+  const Loc l21 = locate<21>(i, a.n, a.soa, a.lw);
+  const Loc l3 = locate<3>(i, a.n, a.soa, a.lw);
+  float p[6], C[21], hc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+  for (int c = 0; c < 6; ++c) p[c] = a.state_in[l6.base + c * l6.stride];
+#pragma unroll
+  for (int e = 0; e < 21; ++e) C[e] = a.cov_in[l21.base + e * l21.stride];
+#pragma unroll
+  for (int c = 0; c < (KIND == kP2z ? 3 : 6); ++c) hc[c] = a.hitcov[l6.base + c * l6.stride];
+  unsigned st = step_in_double<KIND>(
+      p, C, (float)a.charge[i], a.bz, a.surf[a.surf_per_track ? i : 0], a.hit[l3.base],
+      a.hit[l3.base + l3.stride], KIND == kP2z ? 0.0f : a.hit[l3.base + 2 * l3.stride], hc);
+  st |= finite_status(p, C);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) __stcs(a.state_out + l6.base + c * l6.stride, p[c]);
+#pragma unroll
+  for (int e = 0; e < 21; ++e) __stcs(a.cov_out + l21.base + e * l21.stride, C[e]);
+  a.status[i] = (uint8_t)st;
+}
+
 // The redo pass of KF_ADAPTIVE: each block gathers the marked tracks of its
 // span of kRedoSpan tracks (one 16-byte status load per 16 tracks), then its
-// threads run the FP64 step on them, 32 marked tracks to a warp.
+// threads run the FP64 step on them, one each.  (Four warps sharing 32 tracks,
+// as the chain's redo does, does not pay for one step: 2,048-track spans of
+// 300,007 tracks 30.3 against 26.4 us, 20,000: 17.5 against 18.8.)
 template <int KIND>
-__global__ void __launch_bounds__(kRedoThreads) redo_pass_kernel(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(kRedoThreads)
+    redo_pass_kernel(const __grid_constant__ StepArgs a) {
   __shared__ uint16_t list[kRedoSpan];
   __shared__ int count;
   // Launched as a programmatic dependent of the step kernel: wait here until
@@ -193,10 +222,7 @@ __global__ void __launch_bounds__(kRedoThreads) redo_pass_kernel(const __grid_co
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
   const int cnt = gather_marked(a.status, span0, a.n, list, &count);
-  for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
-    const int64_t i = span0 + list[q];
-    a.status[i] = (uint8_t)redo_track_fp64<KIND>(a, i);
-  }
+  for (int q = threadIdx.x; q < cnt; q += blockDim.x) redo_track_fp64<KIND>(a, span0 + list[q]);
 }
 
 int launch_redo_pass(int kind, const StepArgs &a, cudaStream_t s) {

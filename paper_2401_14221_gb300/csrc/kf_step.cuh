@@ -32,43 +32,6 @@ struct StepArgs {
 };
 
 #ifdef __CUDACC__
-// The kAdaptive redo of track i of a step launch: read its inputs from
-// global memory, run the step in double, write its outputs there and return
-// its status (finite check included).  Used by the redo pass, a kernel of its
-// own, so that the FP32 kernel's registers never carry the FP64 step.  In
-// place is safe: the FP32 kernel did not store this track's result.
-template <int KIND>
-__device__ __forceinline__ unsigned redo_track_fp64(const StepArgs &a, int64_t i) {
-  int64_t b6, b21, b3, s;
-  if (a.soa) {
-    b6 = b21 = b3 = i;
-    s = a.n;
-  } else {
-    const int64_t W = int64_t(1) << a.lw, blk = i >> a.lw, r = i & (W - 1);
-    b6 = blk * 6 * W + r;
-    b21 = blk * 21 * W + r;
-    b3 = blk * 3 * W + r;
-    s = W;
-  }
-  float pf[6], Cf[21], hc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-  for (int c = 0; c < 6; ++c) pf[c] = a.state_in[b6 + c * s];
-#pragma unroll
-  for (int e = 0; e < 21; ++e) Cf[e] = a.cov_in[b21 + e * s];
-  constexpr int nhc = KIND == kP2z ? 3 : 6;
-#pragma unroll
-  for (int c = 0; c < nhc; ++c) hc[c] = a.hitcov[b6 + c * s];
-  unsigned st = step_in_double<KIND>(pf, Cf, (float)a.charge[i], a.bz,
-                                     a.surf[a.surf_per_track ? i : 0], a.hit[b3], a.hit[b3 + s],
-                                     KIND == kP2z ? 0.0f : a.hit[b3 + 2 * s], hc);
-  st |= finite_status(pf, Cf);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) __stcs(a.state_out + b6 + c * s, pf[c]);
-#pragma unroll
-  for (int e = 0; e < 21; ++e) __stcs(a.cov_out + b21 + e * s, Cf[e]);
-  return st;
-}
-
 // Status bytes base .. base+15 of an [n] array as four little-endian words:
 // one 16-byte load where the array is 16-byte aligned and the run is whole,
 // byte loads otherwise (bytes at or past n read as 0).
@@ -85,48 +48,32 @@ __device__ __forceinline__ uint4 load_status16(const uint8_t *status, int64_t ba
 // Redo passes gather the marked tracks of a span of kRedoSpan tracks into a
 // shared-memory list before running them, so that each warp runs up to 32
 // marked tracks instead of one marked track among 31 idle lanes: GB300
-// issues an FP64 warp instruction over many cycles whether or not its lanes
-// are active.  The pass is latency-bound (one FP64 warp per scheduler
-// issues on 8 % of cycles), so its time is one warp's chain as long as every
-// marked track runs in the first round: a block has kRedoThreads threads
-// (the double-precision step takes about 190 registers; five 64-thread
-// blocks fit an SM, so the 478 spans of a 1.96 M-track chain are resident
-// at once), and a span is small enough that its marks rarely exceed the
-// block's threads (about 0.6 % of chain tracks are marked: 24 per span on
-// average).  256-thread blocks (one per SM) and 8,192-track spans (48 marks
-// on average, some spans over 64) each took a second round and about
-// doubled the pass.
-constexpr int kRedoSpan = 4096;
-constexpr int kRedoThreads = 64;
+// issues an FP64 warp instruction over 64 cycles whether or not its lanes
+// are active.  A block has one warp per scheduler, and a span is small enough
+// that its marks rarely take it a second round; spans of 2,048 led 1,024 and
+// 4,096 (us per step, 960,000 tracks with nothing marked: 37.1, 38.4, 37.2;
+// 960,000 with 3 % marked: 55, 72, 56; 300,007: 26.4, 26.6, 28.0).
+constexpr int kRedoSpan = 2048;
+constexpr int kRedoThreads = 128;
 
 // Fill list[0..count) with the offsets (from span0) of the tracks marked
 // kRedo among [span0, min(span0 + kRedoSpan, n)); returns the count.  Every
-// thread of the block (kRedoThreads of them) must call it.  Each thread
-// scans kRedoSpan / (16 kRedoThreads) runs of 16 status bytes, striding by
-// the block; all its loads are issued before any is examined, so a span
+// thread of the block must call it; each looks at 16 status bytes, so a span
 // with nothing marked costs one memory latency.
 __device__ __forceinline__ int gather_marked(const uint8_t *status, int64_t span0, int64_t n,
                                              uint16_t *list, int *count) {
-  constexpr int kRuns = kRedoSpan / (16 * kRedoThreads);
-  static_assert(kRuns * 16 * kRedoThreads == kRedoSpan, "whole runs per thread");
+  static_assert(kRedoSpan == 16 * kRedoThreads, "one run of 16 per thread");
   static_assert(kRedoSpan <= 65536, "span offsets are 16-bit");
   constexpr uint32_t kMarks = 0x01010101u * kRedo;  // the kRedo bit of each byte
   if (threadIdx.x == 0) *count = 0;
-  uint4 v[kRuns];
-#pragma unroll
-  for (int r = 0; r < kRuns; ++r) {
-    const int64_t base = span0 + (int64_t)(r * kRedoThreads + threadIdx.x) * 16;
-    v[r] = base < n ? load_status16(status, base, n) : make_uint4(0u, 0u, 0u, 0u);
-  }
+  const int off = (int)threadIdx.x * 16;
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  if (span0 + off < n) v = load_status16(status, span0 + off, n);
   __syncthreads();  // count is 0
-#pragma unroll
-  for (int r = 0; r < kRuns; ++r) {
-    const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-    if (((w[0] | w[1] | w[2] | w[3]) & kMarks) == 0u) continue;
-    const int off = (r * kRedoThreads + threadIdx.x) * 16;
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  if ((w[0] | w[1] | w[2] | w[3]) & kMarks)
     for (int j = 0; j < 16; ++j)
       if ((w[j >> 2] >> (8 * (j & 3))) & kRedo) list[atomicAdd(count, 1)] = (uint16_t)(off + j);
-  }
   __syncthreads();
   return *count;
 }

@@ -131,9 +131,8 @@ __global__ void __launch_bounds__(kRedoThreads)
     const Loc l3 = locate<3>(i, a.n, a.soa, a.lw);
     float pf[6], Cf[21], hc[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
     load_compressed(a, l6, lr, pf, Cf);
-    constexpr int nhc = KIND == kP2z ? 3 : 6;
 #pragma unroll
-    for (int c = 0; c < nhc; ++c) hc[c] = a.hitcov[l6.base + c * l6.stride];
+    for (int c = 0; c < (KIND == kP2z ? 3 : 6); ++c) hc[c] = a.hitcov[l6.base + c * l6.stride];
     unsigned st = step_in_double<KIND>(pf, Cf, (float)a.charge[i], a.bz,
                                        a.surf[a.surf_per_track ? i : 0], a.hit[l3.base],
                                        a.hit[l3.base + l3.stride],
