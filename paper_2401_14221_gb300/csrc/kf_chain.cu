@@ -20,6 +20,7 @@
 #include "kf_device.cuh"
 #include "kf_step.cuh"
 #include "kf_chain.cuh"
+#include "kf_chain_kernel.cuh"
 #include "kf_fp64_group.cuh"
 
 namespace kf {
@@ -28,76 +29,7 @@ namespace staged {
 int sm_count(int dev, int *out);
 }  // namespace staged
 
-struct ChainArgs {
-  float *state;
-  float *cov;
-  const int8_t *charge;
-  const float *hits;     // [L] arrays of 3 components in the layout
-  const float *hitcovs;  // [L] arrays of 6 components in the layout
-  uint8_t *status;
-  int64_t n;
-  int64_t hit_stride;  // floats between consecutive layers' hit arrays
-  int64_t hc_stride;   // floats between consecutive layers' hit-cov arrays
-  int32_t soa;
-  int32_t lw;
-  float bz;
-  int32_t L;
-  int32_t kinds[KF_MAX_LAYERS];
-  float pos[KF_MAX_LAYERS];
-};
-
 namespace {
-
-// Track i of the chain: load, run every layer, store.
-template <int VARIANT>
-__device__ __forceinline__ void chain_one(const ChainArgs &a, int64_t i) {
-  const ChainLoc l6 = chain_locate<6>(i, a.n, a.soa, a.lw);
-  const ChainLoc l21 = chain_locate<21>(i, a.n, a.soa, a.lw);
-  const ChainLoc l3 = chain_locate<3>(i, a.n, a.soa, a.lw);
-
-  float p[6], C[21];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) p[c] = a.state[l6.base + c * l6.stride];
-#pragma unroll
-  for (int e = 0; e < 21; ++e) C[e] = a.cov[l21.base + e * l21.stride];
-  const float qf = (float)__ldg(a.charge + i);
-
-  unsigned st;
-  if constexpr (VARIANT == kAdaptive) {
-    st = chain_track_marking(p, C, qf, a.bz, a.L, a.kinds, a.pos, a.hits, a.hit_stride, a.hitcovs,
-                             a.hc_stride, l3, l6);
-    if (st & kRedo) {  // left to chain_redo_kernel, inputs untouched
-      a.status[i] = (uint8_t)kRedo;
-      return;
-    }
-  } else if constexpr (VARIANT == kFP64) {
-    st = chain_track_fp64(p, C, qf, a.bz, a.L, a.kinds, a.pos, a.hits, a.hit_stride, a.hitcovs,
-                          a.hc_stride, l3, l6);
-  } else {
-    st = chain_track<VARIANT>(p, C, qf, a.bz, a.L, a.kinds, a.pos, a.hits, a.hit_stride,
-                              a.hitcovs, a.hc_stride, l3, l6);
-  }
-  st |= finite_status(p, C);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) a.state[l6.base + c * l6.stride] = p[c];
-#pragma unroll
-  for (int e = 0; e < 21; ++e) a.cov[l21.base + e * l21.stride] = C[e];
-  if (a.status) a.status[i] = (uint8_t)st;
-}
-
-template <int VARIANT>
-__global__ void __launch_bounds__(256) chain_kernel(const ChainArgs a) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < a.n) chain_one<VARIANT>(a, i);
-}
-
-// KF_ADAPTIVE's first pass, held to 80 registers so that three 256-thread
-// CTAs fit an SM (unbounded it takes 96: two CTAs; measured on the 256-event
-// chain workload, the adaptive chain 1.057 -> 0.949 ms, no spills).
-__global__ void __launch_bounds__(256, 3) chain_mark_kernel(const ChainArgs a) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < a.n) chain_one<kAdaptive>(a, i);
-}
 
 // KF_ADAPTIVE's second pass for one marked track: the whole chain again
 // from its (untouched) inputs, in double (chain_track_fp64).
@@ -329,7 +261,17 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   a.lw = d.lw;
   a.bz = params->bz;
   a.L = L;
-  LaunchConfig cfg{KF_STEP_DIRECT, 256, 0};
+  int dev = 0, sms = 0;
+  if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
+  if (int rc = staged::sm_count(dev, &sms)) return rc;
+  // CTA size: 64 threads spread a small batch over the SMs and waste least in
+  // the last wave (us with 64, 128, 256 threads: FP32 5,000 tracks 15.0, 15.0,
+  // 17.1, 440,000: 107, 107, 111; FP64 update 60,000: 144, 160, 160; KF_FP64
+  // 20,000: 250, 322, 320).  The double-float update leads with 256 once the
+  // device is full (60,000: 54.9, 53.9, 51.9; 1.75 M: 1,118, 1,102, 1,010) and
+  // with 128 before (5,000: 31.4, 29.3, 33.4).
+  const int df_threads = d.n > (int64_t)128 * sms ? 256 : 128;
+  LaunchConfig cfg{KF_STEP_DIRECT, params->precision == KF_DF_UPDATE ? df_threads : 64, 0};
   if (const LaunchConfig *o = thread_override()) {
     cfg = *o;
   } else {
@@ -340,24 +282,22 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   const int64_t blocks = (d.n + threads - 1) / threads;
   if (blocks > 0x7fffffffLL) return set_error(KF_ERR_ARG, "n too large for one launch");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (params->precision == KF_FP64) {  // few tracks: four warps to 32 of them
-    int dev = 0, sms = 0;
-    if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
-    if (int rc = staged::sm_count(dev, &sms)) return rc;
-    if (d.n <= (int64_t)sms * kGroupTracksPerSm) {
-      chain_group_kernel<<<(unsigned)((d.n + 31) / 32), kRedoThreads, 0, s>>>(a);
-      return check_cuda(cudaGetLastError(), "chain launch");
-    }
+  if (params->precision == KF_FP64 && d.n <= (int64_t)sms * kGroupTracksPerSm) {
+    chain_group_kernel<<<(unsigned)((d.n + 31) / 32), kRedoThreads, 0, s>>>(a);
+    return check_cuda(cudaGetLastError(), "chain launch");
   }
+  const unsigned g = (unsigned)blocks;
+  int rc = KF_OK;
   switch (params->precision) {
-    case KF_FP32: chain_kernel<kFP32><<<(unsigned)blocks, threads, 0, s>>>(a); break;
-    case KF_FP64_UPDATE: chain_kernel<kFP64Update><<<(unsigned)blocks, threads, 0, s>>>(a); break;
-    case KF_JOSEPH: chain_kernel<kJoseph><<<(unsigned)blocks, threads, 0, s>>>(a); break;
-    case KF_FP64: chain_kernel<kFP64><<<(unsigned)blocks, threads, 0, s>>>(a); break;
-    case KF_DF_UPDATE: chain_kernel<kDFUpdate><<<(unsigned)blocks, threads, 0, s>>>(a); break;
-    default: chain_mark_kernel<<<(unsigned)blocks, threads, 0, s>>>(a); break;
+    case KF_FP32: rc = launch_chain_fp32(a, g, threads, s); break;
+    case KF_ADAPTIVE: rc = launch_chain_mark(a, g, threads, s); break;
+    case KF_FP64_UPDATE: chain_kernel<kFP64Update, 0><<<g, threads, 0, s>>>(a); break;
+    case KF_JOSEPH: rc = launch_chain_joseph(a, g, threads, s); break;
+    case KF_FP64: chain_kernel<kFP64, 0><<<g, threads, 0, s>>>(a); break;
+    default: chain_kernel<kDFUpdate, 0><<<g, threads, 0, s>>>(a); break;
   }
-  if (int rc = check_cuda(cudaGetLastError(), "chain launch")) return rc;
+  if (rc != KF_OK) return rc;
+  if (int rc2 = check_cuda(cudaGetLastError(), "chain launch")) return rc2;
   if (params->precision != KF_ADAPTIVE) return KF_OK;
   return launch_chain_redo(a, s);
 }

@@ -304,3 +304,28 @@ def test_adaptive_chain_redo_pass(dev, chain_full):
         kf.kf_kalman_chain(kf.make_params(cw.bz, kf.KF_ADAPTIVE), dc.layout, dc.state, dc.cov,
                            dc.charge, dc.hits, dc.hit_covs, dc.layers, None)
     assert e.value.code == kf.KF_ERR_ARG
+
+
+@pytest.mark.parametrize("precision", [kf.KF_FP32, kf.KF_JOSEPH, kf.KF_ADAPTIVE, kf.KF_DF_UPDATE])
+@pytest.mark.parametrize("n", [1, 63, 333])
+def test_chain_kernels_of_every_layout_agree_bitwise(dev, n, precision):
+    # a kernel per layout (the block width known at compile time), the same
+    # arithmetic: equal results, and equal to the per-layer launches where the
+    # state is FP32 between layers (AoSoA: a layer's hits of an SoA array are
+    # 16-byte aligned, as a single step wants them, only for some n)
+    cw = W.make_chain(events=1, seed=17, sizes=np.array([n]), pool=256)
+    got = []
+    for layout, width in [(kf.KF_SOA, 0)] + [(kf.KF_AOSOA, w) for w in (16, 32, 64, 128)]:
+        dc = kf.chain_upload(cw, layout, width, dev)
+        dc.run(precision)
+        torch.cuda.synchronize()
+        got.append(dc.download())
+        if layout == kf.KF_AOSOA and precision != kf.KF_ADAPTIVE:
+            dc.reset()
+            dc.run_plain(precision)
+            torch.cuda.synchronize()
+            plain = dc.download()
+            assert np.array_equal(got[-1][0], plain[0]) and np.array_equal(got[-1][1], plain[1])
+    for other in got[1:]:
+        for a, b in zip(got[0], other):
+            assert np.array_equal(a, b)
