@@ -268,8 +268,8 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   // the last wave (us with 64, 128, 256 threads: FP32 5,000 tracks 15.0, 15.0,
   // 17.1, 440,000: 107, 107, 111; FP64 update 60,000: 144, 160, 160; KF_FP64
   // 20,000: 250, 322, 320).  The double-float update leads with 256 once the
-  // device is full (60,000: 54.9, 53.9, 51.9; 1.75 M: 1,118, 1,102, 1,010) and
-  // with 128 before (5,000: 31.4, 29.3, 33.4).
+  // device is full (60,000: 45.7, 45.7, 43.6; 1.75 M: 899, 889, 834) and with
+  // 128 before (5,000: 25.2, 25.2, 27.3).
   const int df_threads = d.n > (int64_t)128 * sms ? 256 : 128;
   LaunchConfig cfg{KF_STEP_DIRECT, params->precision == KF_DF_UPDATE ? df_threads : 64, 0};
   if (const LaunchConfig *o = thread_override()) {

@@ -84,12 +84,9 @@ __device__ __forceinline__ bool has_bit_(unsigned st, unsigned b) { return (st &
 //   add_dd        Joldes, Muller, Popescu, ACM TOMS 44 (2017) art. 15,
 //                 Algorithm 6 (accurate double-word + double-word), relative
 //                 error <= 3u^2 / (1 - 4u)
-//   add_df        ibid., Algorithm 4 (double-word + float), <= 2u^2
 //   mul_df        ibid., Algorithm 9 (double-word x float with an FMA), <= 2u^2
-//   mul_dd        ibid., Algorithm 12 (double-word x double-word with FMAs),
-//                 <= 4u^2
-//   rcp_d         one Newton-Raphson step x0 + x0 (1 - y x0) from the
-//                 correctly rounded float reciprocal x0 of y's leading part
+//   rcp_d         one Newton-Raphson step x0 + x0 (1 - y x0) from the float
+//                 reciprocal x0 of y's leading part
 //   dot2_df       a x + b y as a compensated dot product (below)
 // Every step is an explicitly rounded float operation, so no compiler
 // contraction can break an error-free transformation.
@@ -117,31 +114,21 @@ __device__ __forceinline__ dfl add_dd(dfl x, dfl y) {
   const dfl v = fast_two_sum(s.hi, __fadd_rn(s.lo, t.hi));
   return fast_two_sum(v.hi, __fadd_rn(t.lo, v.lo));
 }
-__device__ __forceinline__ dfl add_df(dfl x, float y) {
-  const dfl s = two_sum(x.hi, y);
-  return fast_two_sum(s.hi, __fadd_rn(x.lo, s.lo));
-}
 __device__ __forceinline__ dfl mul_df(dfl x, float y) {
   const dfl c = two_prod(x.hi, y);
   return fast_two_sum(c.hi, __fmaf_rn(x.lo, y, c.lo));
 }
-__device__ __forceinline__ dfl mul_dd(dfl x, dfl y) {
-  const dfl c = two_prod(x.hi, y.hi);
-  const float t0 = __fmul_rn(x.lo, y.lo);
-  const float t1 = __fmaf_rn(x.hi, y.lo, t0);
-  const float c2 = __fmaf_rn(x.lo, y.hi, t1);
-  return fast_two_sum(c.hi, __fadd_rn(c.lo, c2));
-}
 __device__ __forceinline__ dfl neg_d(dfl x) { return {-x.hi, -x.lo}; }
 __device__ __forceinline__ dfl rcp_d(dfl y) {
-  const float x0 = __frcp_rn(y.hi);
+  // x0: the approximate reciprocal (within 1 ulp) after a step of its own,
+  // within half an ulp and 2^-46
+  float a;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(y.hi));
+  const float x0 = __fmaf_rn(a, __fmaf_rn(-y.hi, a, 1.0f), a);
   const dfl p = mul_df(y, x0);                       // y x0 = 1 - e, p.hi within ulps of 1
   const float e = __fsub_rn(__fsub_rn(1.0f, p.hi), p.lo);  // 1 - p.hi is exact
   return fast_two_sum(x0, __fmul_rn(x0, e));
 }
-// The float nearest to hi + lo.
-__device__ __forceinline__ float to_float(dfl x) { return __fadd_rn(x.hi, x.lo); }
-
 // a x + b y for double-word a, b and floats x, y, as a compensated dot
 // product (the structure of Algorithm Dot2 of Ogita, Rump and Oishi, SIAM
 // J. Sci. Comput. 26 (2005) 1955): the leading products and their sum are
@@ -158,17 +145,40 @@ __device__ __forceinline__ dfl dot2_df(dfl a, float x, dfl b, float y) {
   return fast_two_sum(s.hi, __fadd_rn(t, s.lo));
 }
 
-// c - (a x + b y) the same way, with the float c taken into the error-free
+// a x + b y rounded to float: the same without the renormalisation, whose
+// leading part the one rounding gives.
+__device__ __forceinline__ float dot2_df_to_float(dfl a, float x, dfl b, float y) {
+  const dfl p = two_prod(a.hi, x), q = two_prod(b.hi, y);
+  const dfl s = two_sum(p.hi, q.hi);
+  float t = __fadd_rn(p.lo, q.lo);
+  t = __fmaf_rn(a.lo, x, t);
+  t = __fmaf_rn(b.lo, y, t);
+  return __fadd_rn(s.hi, __fadd_rn(t, s.lo));
+}
+
+// The same of double-word x and y.
+__device__ __forceinline__ float dot2_dd_to_float(dfl a, dfl x, dfl b, dfl y) {
+  const dfl p = two_prod(a.hi, x.hi), q = two_prod(b.hi, y.hi);
+  const dfl s = two_sum(p.hi, q.hi);
+  float t = __fadd_rn(p.lo, q.lo);
+  t = __fmaf_rn(a.lo, x.hi, t);
+  t = __fmaf_rn(a.hi, x.lo, t);
+  t = __fmaf_rn(b.lo, y.hi, t);
+  t = __fmaf_rn(b.hi, y.lo, t);
+  return __fadd_rn(s.hi, __fadd_rn(t, s.lo));
+}
+
+// c + a x + b y rounded to float, with the float c taken into the error-free
 // sum.
-__device__ __forceinline__ dfl sub_dot2_df(float c, dfl a, float x, dfl b, float y) {
-  const dfl p = two_prod(-a.hi, x), q = two_prod(-b.hi, y);
+__device__ __forceinline__ float add_dot2_df(float c, dfl a, float x, dfl b, float y) {
+  const dfl p = two_prod(a.hi, x), q = two_prod(b.hi, y);
   const dfl s1 = two_sum(p.hi, q.hi);
   const dfl s2 = two_sum(s1.hi, c);
   float t = __fadd_rn(p.lo, q.lo);
-  t = __fmaf_rn(-a.lo, x, t);
-  t = __fmaf_rn(-b.lo, y, t);
+  t = __fmaf_rn(a.lo, x, t);
+  t = __fmaf_rn(b.lo, y, t);
   t = __fadd_rn(t, s1.lo);
-  return fast_two_sum(s2.hi, __fadd_rn(t, s2.lo));
+  return __fadd_rn(s2.hi, __fadd_rn(t, s2.lo));
 }
 
 // =============================================================== traits
