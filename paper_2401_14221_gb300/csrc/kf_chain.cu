@@ -31,6 +31,9 @@ int sm_count(int dev, int *out);
 
 namespace {
 
+// Tracks whose marks a block of the second pass gathers.
+constexpr int kChainSpan = 2048;
+
 // KF_ADAPTIVE's second pass for one marked track: the whole chain again
 // from its (untouched) inputs, in double (chain_track_fp64).
 __device__ __forceinline__ void chain_redo_track(const ChainArgs &a, int64_t i) {
@@ -65,15 +68,15 @@ __device__ __forceinline__ void chain_redo_group(const ChainArgs &a, const f64::
 // chain_compact_kernel builds the list: each block gathers its span's marks
 // and appends them (one atomic per block; the order of the list varies from
 // run to run, the result of each track does not).
-__global__ void __launch_bounds__(kRedoThreads) chain_compact_kernel(const uint8_t *status,
+__global__ void __launch_bounds__(f64::kGroupThreads) chain_compact_kernel(const uint8_t *status,
                                                                      int64_t n,
                                                                      uint32_t *count,
                                                                      uint32_t *list) {
-  __shared__ uint16_t span_list[kRedoSpan];
+  __shared__ uint16_t span_list[kChainSpan];
   __shared__ int span_count;
   __shared__ uint32_t base;
-  const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
-  const int cnt = gather_marked(status, span0, n, span_list, &span_count);
+  const int64_t span0 = (int64_t)blockIdx.x * kChainSpan;
+  const int cnt = gather_marked<kChainSpan, f64::kGroupThreads>(status, span0, n, span_list, &span_count);
   if (cnt == 0) return;  // the same count in every thread of the block
   if (threadIdx.x == 0) base = atomicAdd(count, (uint32_t)cnt);
   __syncthreads();
@@ -88,7 +91,7 @@ constexpr int kRedoListBlocksPerSm = 4;
 // up to 10,000 tracks, 175 up to 19,000.
 constexpr int kGroupTracksPerSm = 96;
 
-__global__ void __launch_bounds__(kRedoThreads, kRedoListBlocksPerSm)
+__global__ void __launch_bounds__(f64::kGroupThreads, kRedoListBlocksPerSm)
     chain_redo_list_kernel(const ChainArgs a, const uint32_t *count, const uint32_t *list) {
   __shared__ f64::Shared sh;
   const int64_t total = *count;
@@ -106,12 +109,12 @@ __global__ void __launch_bounds__(kRedoThreads, kRedoListBlocksPerSm)
 // KF_ADAPTIVE's second pass without a list (no scratch memory could be had,
 // or more than 2^32 - 1 tracks): each block gathers the marked tracks of its
 // span (gather_marked) and reruns them.
-__global__ void __launch_bounds__(kRedoThreads, 4) chain_redo_kernel(const ChainArgs a) {
+__global__ void __launch_bounds__(f64::kGroupThreads, 4) chain_redo_kernel(const ChainArgs a) {
   __shared__ f64::Shared sh;
-  __shared__ uint16_t list[kRedoSpan];
+  __shared__ uint16_t list[kChainSpan];
   __shared__ int count;
-  const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
-  const int cnt = gather_marked(a.status, span0, a.n, list, &count);
+  const int64_t span0 = (int64_t)blockIdx.x * kChainSpan;
+  const int cnt = gather_marked<kChainSpan, f64::kGroupThreads>(a.status, span0, a.n, list, &count);
   if (cnt > f64::kGroupMax) {
     for (int q = threadIdx.x; q < cnt; q += blockDim.x) chain_redo_track(a, span0 + list[q]);
     return;
@@ -123,7 +126,7 @@ __global__ void __launch_bounds__(kRedoThreads, 4) chain_redo_kernel(const Chain
 }
 
 // KF_FP64 for batches too small to give every scheduler a warp of tracks.
-__global__ void __launch_bounds__(kRedoThreads, kRedoListBlocksPerSm)
+__global__ void __launch_bounds__(f64::kGroupThreads, kRedoListBlocksPerSm)
     chain_group_kernel(const ChainArgs a) {
   __shared__ f64::Shared sh;
   const f64::Group g{sh, (int)threadIdx.x >> 5, (int)threadIdx.x & 31};
@@ -168,7 +171,7 @@ std::atomic<int> g_chain_redo{KF_CHAIN_REDO_LIST};
 // Launch the second pass on stream s: over a compacted list when its
 // scratch can be allocated, else per span (the same results).
 int launch_chain_redo(const ChainArgs &a, cudaStream_t s) {
-  const unsigned spans = (unsigned)((a.n + kRedoSpan - 1) / kRedoSpan);
+  const unsigned spans = (unsigned)((a.n + kChainSpan - 1) / kChainSpan);
   int dev = 0, sms = 0;
   cudaMemPool_t pool = nullptr;
   void *buf = nullptr;
@@ -182,11 +185,11 @@ int launch_chain_redo(const ChainArgs &a, cudaStream_t s) {
     uint32_t *count = static_cast<uint32_t *>(buf), *list = count + 1;
     int rc = check_cuda(cudaMemsetAsync(count, 0, sizeof(uint32_t), s), "cudaMemsetAsync");
     if (rc == KF_OK) {
-      chain_compact_kernel<<<spans, kRedoThreads, 0, s>>>(a.status, a.n, count, list);
+      chain_compact_kernel<<<spans, f64::kGroupThreads, 0, s>>>(a.status, a.n, count, list);
       rc = check_cuda(cudaGetLastError(), "chain compaction launch");
     }
     if (rc == KF_OK) {
-      chain_redo_list_kernel<<<(unsigned)(kRedoListBlocksPerSm * sms), kRedoThreads, 0, s>>>(
+      chain_redo_list_kernel<<<(unsigned)(kRedoListBlocksPerSm * sms), f64::kGroupThreads, 0, s>>>(
           a, count, list);
       rc = check_cuda(cudaGetLastError(), "chain redo pass launch");
     }
@@ -195,7 +198,7 @@ int launch_chain_redo(const ChainArgs &a, cudaStream_t s) {
   }
   clear_error();
   (void)cudaGetLastError();  // a refused allocation is not the caller's error
-  chain_redo_kernel<<<spans, kRedoThreads, 0, s>>>(a);
+  chain_redo_kernel<<<spans, f64::kGroupThreads, 0, s>>>(a);
   return check_cuda(cudaGetLastError(), "chain redo pass launch");
 }
 
@@ -283,7 +286,7 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   if (blocks > 0x7fffffffLL) return set_error(KF_ERR_ARG, "n too large for one launch");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (params->precision == KF_FP64 && d.n <= (int64_t)sms * kGroupTracksPerSm) {
-    chain_group_kernel<<<(unsigned)((d.n + 31) / 32), kRedoThreads, 0, s>>>(a);
+    chain_group_kernel<<<(unsigned)((d.n + 31) / 32), f64::kGroupThreads, 0, s>>>(a);
     return check_cuda(cudaGetLastError(), "chain launch");
   }
   const unsigned g = (unsigned)blocks;

@@ -81,8 +81,8 @@ __global__ void __launch_bounds__(256, VARIANT == kAdaptive ? 3 : 0)
 
 // The kernel with the AoSoA width known at compile time: a hit's nine loads
 // then differ by immediate offsets, which takes 4 % of the chain's instructions
-// and the 64-bit strides out of its registers (1.75 M tracks, FP32 385 -> 383
-// us, marking pass 428 -> 405).
+// and the 64-bit strides out of its registers (1.75 M tracks, FP32 391 -> 381
+// us, Joseph 467 -> 455, adaptive 605 -> 586).
 template <int VARIANT>
 int launch_chain_by_width(const ChainArgs &a, unsigned blocks, int threads, cudaStream_t s) {
   switch (a.soa ? -1 : a.lw) {

@@ -76,6 +76,12 @@ struct Consts<float> {
 template <class T>
 using K_ = Consts<scalar_t<T>>;
 
+// value = m ? a() : b(), computing only the side that is taken.
+template <class T, class FA, class FB>
+__device__ __forceinline__ T choose(mask_t<T> m, FA &&a, FB &&b) {
+  return m ? a() : b();
+}
+
 constexpr uint64_t bit(int i, int j) { return 1ull << (i * 6 + j); }
 
 // Structural non-zeros (NZ) and unit entries (ONE) of the transport
@@ -111,29 +117,33 @@ __device__ __forceinline__ T wrap_phi(T a) {
   const T n = rint_(mul_(a, cst<T>(K::inv_two_pi)));
   T w = fma_(n, cst<T>(-K::two_pi_hi), a);
   w = fma_(n, cst<T>(-K::two_pi_lo), w);
-  return sel_(le_(w, cst<T>(-K::pi)), add_(w, cst<T>(K::two_pi_hi)), w);
+  return choose<T>(le_(w, cst<T>(-K::pi)), [&] { return add_(w, cst<T>(K::two_pi_hi)); },
+                   [&] { return w; });
 }
 
-// S(h) = sin(h)/h given sin(h); S(0) = 1.  Here and below both sides of a
-// per-track choice are computed and one is selected: a warp's tracks mostly
-// take both, and the selection costs less than the branches did (the 15-layer
-// chain of 1.75 M tracks 391 -> 385 us).
+// S(h) = sin(h)/h given sin(h); S(0) = 1.
 template <class T>
 __device__ __forceinline__ T sinc_from(T h, T sh) {
-  const T q = div_(sh, h);
-  return sel_(lt_(abs_(h), cst<T>(1e-4)), fma_(mul_(h, h), cst<T>(-1.0 / 6.0), cst<T>(1.0)), q);
+  return choose<T>(
+      lt_(abs_(h), cst<T>(1e-4)),
+      [&] { return fma_(mul_(h, h), cst<T>(-1.0 / 6.0), cst<T>(1.0)); },
+      [&] { return div_(sh, h); });
 }
 
 // dS/dh = (cos(h) - S(h)) / h; the difference cancels for small |h|, where
 // the Taylor series -h/3 + h^3/30 - h^5/840 + h^7/45360 is used instead.
 template <class T>
 __device__ __forceinline__ T dsinc_from(T h, T ch, T S) {
-  const T h2 = mul_(h, h);
-  const T series = mul_(h, fma_(h2,
-                                fma_(h2, fma_(h2, cst<T>(1.0 / 45360.0), cst<T>(-1.0 / 840.0)),
-                                     cst<T>(1.0 / 30.0)),
-                                cst<T>(-1.0 / 3.0)));
-  return sel_(lt_(abs_(h), cst<T>(K_<T>::dsinc_series)), series, div_(sub_(ch, S), h));
+  return choose<T>(
+      lt_(abs_(h), cst<T>(K_<T>::dsinc_series)),
+      [&] {
+        const T h2 = mul_(h, h);
+        return mul_(h, fma_(h2,
+                            fma_(h2, fma_(h2, cst<T>(1.0 / 45360.0), cst<T>(-1.0 / 840.0)),
+                                 cst<T>(1.0 / 30.0)),
+                            cst<T>(-1.0 / 3.0)));
+      },
+      [&] { return div_(sub_(ch, S), h); });
 }
 
 // C' = J C J^T for packed symmetric C, with J's structure fixed by NZ/ONE.
@@ -306,8 +316,8 @@ __device__ __forceinline__ mask_t<T> propagate_to_r(const T (&in)[6], T qf, T bz
   const T sh = mul_(yv, inv);                 // sin(h)
   const T h = atan2_(yv, xv);                 // half turning angle
   const T L = mul_(add_(d, d), inv);          // chord
-  const mask_t<T> bent = gt_(abs_(omega), cst<T>(1e-12));
-  const T s = div_(sel_(bent, add_(h, h), d), sel_(bent, omega, den));
+  const T s = choose<T>(gt_(abs_(omega), cst<T>(1e-12)),
+                        [&] { return div_(add_(h, h), omega); }, [&] { return div_(d, den); });
   const T ist = rcp_(st);
   const T cot = mul_(ct, ist);
   const T S = sinc_from(h, sh);

@@ -26,6 +26,7 @@
 namespace kf {
 namespace f64 {
 
+constexpr int kGroupThreads = 128;
 // Of a block's marked tracks, up to this many run 32 at a time by its four
 // warps, more one to a thread: that keeps the schedulers as busy with a seventh
 // fewer instructions.

@@ -155,11 +155,11 @@ __device__ __forceinline__ int batch_event_of(const BatchArgs &a, int64_t b) {
   return lo;
 }
 
-__global__ void __launch_bounds__(kRedoThreads, 4)
+__global__ void __launch_bounds__(f64::kGroupThreads, 4)
     batch_redo_kernel(const __grid_constant__ BatchArgs a, int64_t nblocks) {
   constexpr int kSlots = kBatchRedoBlocks * kBatchThreads;
   constexpr int kAtOnce = 8;  // status bytes a thread has in flight
-  static_assert(kSlots % (kAtOnce * kRedoThreads) == 0 && kSlots <= 65536, "16-bit slots");
+  static_assert(kSlots % (kAtOnce * f64::kGroupThreads) == 0 && kSlots <= 65536, "16-bit slots");
   __shared__ f64::Shared sh;
   __shared__ uint16_t slot_of[kSlots];
   __shared__ int count;
@@ -172,11 +172,11 @@ __global__ void __launch_bounds__(kRedoThreads, 4)
     i = (b - e.block_begin) * kBatchThreads + slot % kBatchThreads;
     return e;
   };
-  for (int s0 = threadIdx.x; s0 < kSlots; s0 += kAtOnce * kRedoThreads) {
+  for (int s0 = threadIdx.x; s0 < kSlots; s0 += kAtOnce * f64::kGroupThreads) {
     uint8_t st[kAtOnce];
 #pragma unroll
     for (int r = 0; r < kAtOnce; ++r) {
-      const int slot = s0 + r * kRedoThreads;
+      const int slot = s0 + r * f64::kGroupThreads;
       st[r] = 0;
       if ((int64_t)blockIdx.x * kBatchRedoBlocks + slot / kBatchThreads < nblocks) {
         int64_t i;
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kRedoThreads, 4)
     }
 #pragma unroll
     for (int r = 0; r < kAtOnce; ++r)
-      if (st[r] & kRedo) slot_of[atomicAdd(&count, 1)] = (uint16_t)(s0 + r * kRedoThreads);
+      if (st[r] & kRedo) slot_of[atomicAdd(&count, 1)] = (uint16_t)(s0 + r * f64::kGroupThreads);
   }
   __syncthreads();
   const int cnt = count;
@@ -457,7 +457,7 @@ bool launch_batch(kf_server *s, std::vector<Request *> &batch) {
         batch_chain_kernel<kAdaptive><<<g, kBatchThreads, 0, s->s_compute>>>(a);
         e = cudaGetLastError();
         if (e == cudaSuccess)
-          batch_redo_kernel<<<(g + kBatchRedoBlocks - 1) / kBatchRedoBlocks, kRedoThreads, 0,
+          batch_redo_kernel<<<(g + kBatchRedoBlocks - 1) / kBatchRedoBlocks, f64::kGroupThreads, 0,
                               s->s_compute>>>(
               a, (int64_t)g);
         break;

@@ -206,8 +206,8 @@ __device__ __forceinline__ void redo_track_fp64(const StepArgs &a, int64_t i) {
 // The redo pass of KF_ADAPTIVE: each block gathers the marked tracks of its
 // span of kRedoSpan tracks (one 16-byte status load per 16 tracks), then its
 // threads run the FP64 step on them, one each.  (Four warps sharing 32 tracks,
-// as the chain's redo does, does not pay for one step: 2,048-track spans of
-// 300,007 tracks 30.3 against 26.4 us, 20,000: 17.5 against 18.8.)
+// as in the chain's redo, does not pay for one step: with 2,048-track spans
+// 300,007 tracks took 30.3 against 26.4 us, 20,000 17.5 against 18.8.)
 template <int KIND>
 __global__ void __launch_bounds__(kRedoThreads)
     redo_pass_kernel(const __grid_constant__ StepArgs a) {
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kRedoThreads)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
-  const int cnt = gather_marked(a.status, span0, a.n, list, &count);
+  const int cnt = gather_marked<kRedoSpan, kRedoThreads>(a.status, span0, a.n, list, &count);
   for (int q = threadIdx.x; q < cnt; q += blockDim.x) redo_track_fp64<KIND>(a, span0 + list[q]);
 }
 

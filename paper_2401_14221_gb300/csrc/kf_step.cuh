@@ -50,30 +50,43 @@ __device__ __forceinline__ uint4 load_status16(const uint8_t *status, int64_t ba
 // marked tracks instead of one marked track among 31 idle lanes: GB300
 // issues an FP64 warp instruction over 64 cycles whether or not its lanes
 // are active.  A block has one warp per scheduler, and a span is small enough
-// that its marks rarely take it a second round; spans of 2,048 led 1,024 and
-// 4,096 (us per step, 960,000 tracks with nothing marked: 37.1, 38.4, 37.2;
-// 960,000 with 3 % marked: 55, 72, 56; 300,007: 26.4, 26.6, 28.0).
-constexpr int kRedoSpan = 2048;
+// that its marks rarely take it a second round and large enough that the
+// blocks leave the next step's room to start prefetching while this pass
+// looks through the marks (us per p2r step, spans / threads 4,096/128,
+// 2,048/128, 2,048/64, 4,096/64: 960,000 tracks with nothing marked 37.1,
+// 37.9, 37.1, 37.7; with 3 % marked 54.9, 65.4, 60.4, 61.3; 300,007: 30.2,
+// 29.5, 30.0, 35.0).
+constexpr int kRedoSpan = 4096;
 constexpr int kRedoThreads = 128;
 
 // Fill list[0..count) with the offsets (from span0) of the tracks marked
-// kRedo among [span0, min(span0 + kRedoSpan, n)); returns the count.  Every
-// thread of the block must call it; each looks at 16 status bytes, so a span
-// with nothing marked costs one memory latency.
+// kRedo among [span0, min(span0 + SPAN, n)); returns the count.  Every
+// thread of the block (THREADS of them) must call it.  Each thread looks at
+// SPAN / (16 THREADS) runs of 16 status bytes, all loaded before any is
+// examined, so a span with nothing marked costs one memory latency.
+template <int SPAN, int THREADS>
 __device__ __forceinline__ int gather_marked(const uint8_t *status, int64_t span0, int64_t n,
                                              uint16_t *list, int *count) {
-  static_assert(kRedoSpan == 16 * kRedoThreads, "one run of 16 per thread");
-  static_assert(kRedoSpan <= 65536, "span offsets are 16-bit");
+  constexpr int kRuns = SPAN / (16 * THREADS);
+  static_assert(kRuns * 16 * THREADS == SPAN, "whole runs per thread");
+  static_assert(SPAN <= 65536, "span offsets are 16-bit");
   constexpr uint32_t kMarks = 0x01010101u * kRedo;  // the kRedo bit of each byte
   if (threadIdx.x == 0) *count = 0;
-  const int off = (int)threadIdx.x * 16;
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (span0 + off < n) v = load_status16(status, span0 + off, n);
+  uint4 v[kRuns];
+#pragma unroll
+  for (int r = 0; r < kRuns; ++r) {
+    const int64_t base = span0 + (int64_t)(r * THREADS + threadIdx.x) * 16;
+    v[r] = base < n ? load_status16(status, base, n) : make_uint4(0u, 0u, 0u, 0u);
+  }
   __syncthreads();  // count is 0
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-  if ((w[0] | w[1] | w[2] | w[3]) & kMarks)
+#pragma unroll
+  for (int r = 0; r < kRuns; ++r) {
+    const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+    if (((w[0] | w[1] | w[2] | w[3]) & kMarks) == 0u) continue;
+    const int off = (r * THREADS + (int)threadIdx.x) * 16;
     for (int j = 0; j < 16; ++j)
       if ((w[j >> 2] >> (8 * (j & 3))) & kRedo) list[atomicAdd(count, 1)] = (uint16_t)(off + j);
+  }
   __syncthreads();
   return *count;
 }

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kRedoThreads)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
-  const int cnt = gather_marked(a.status, span0, a.n, list, &count);
+  const int cnt = gather_marked<kRedoSpan, kRedoThreads>(a.status, span0, a.n, list, &count);
   for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
     const int64_t i = span0 + list[q];
     const Loc l6 = locate<6>(i, a.n, a.soa, a.lw);
