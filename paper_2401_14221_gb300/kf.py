@@ -181,8 +181,24 @@ def _ptr(t, name: str, dtype: Optional[torch.dtype] = None):
     return t.data_ptr()
 
 
+_F32, _I8, _U8, _F16 = torch.float32, torch.int8, torch.uint8, torch.float16
+
+
+def _dptr(t, name: str, dtype: torch.dtype):
+    """_ptr for the common argument, a plain contiguous CUDA tensor of the
+    expected type, at a third of its cost; anything else is left to _ptr."""
+    if type(t) is torch.Tensor and t.is_cuda and t.dtype is dtype and t.is_contiguous():
+        return t.data_ptr()
+    return _ptr(t, name, dtype)
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch._C._cuda_getDevice())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
@@ -204,16 +220,15 @@ def make_params(bz: float, precision: int = KF_FP32, flags: int = 0) -> kf_param
 
 def _step(fn_name, params, layout, state_in, cov_in, state_out, cov_out, charge, hit, hit_cov,
           surf, surf_per_track, status, stream):
-    lib = load()
-    f32, i8, u8 = torch.float32, torch.int8, torch.uint8
-    rc = getattr(lib, fn_name)(
+    rc = getattr(_lib or load(), fn_name)(
         ctypes.byref(params), layout,
-        _ptr(state_in, "state_in", f32), _ptr(cov_in, "cov_in", f32),
-        _ptr(state_out, "state_out", f32), _ptr(cov_out, "cov_out", f32),
-        _ptr(charge, "charge", i8), _ptr(hit, "hit", f32), _ptr(hit_cov, "hit_cov", f32),
-        _ptr(surf, "surf", f32), int(surf_per_track), _ptr(status, "status", u8),
+        _dptr(state_in, "state_in", _F32), _dptr(cov_in, "cov_in", _F32),
+        _dptr(state_out, "state_out", _F32), _dptr(cov_out, "cov_out", _F32),
+        _dptr(charge, "charge", _I8), _dptr(hit, "hit", _F32), _dptr(hit_cov, "hit_cov", _F32),
+        _dptr(surf, "surf", _F32), int(surf_per_track), _dptr(status, "status", _U8),
         _stream(stream))
-    _check(rc)
+    if rc != KF_OK:
+        _check(rc)
 
 
 def kf_p2z_propagate_update(params, layout, state_in, cov_in, state_out, cov_out, charge, hit,
@@ -349,29 +364,28 @@ def make_layers(kinds, pos):
 def kf_kalman_chain(params, layout, state, cov, charge, hits, hit_covs, layers, status=None,
                     stream=None):
     """C-ABI kf_kalman_chain (in place on state/cov); `layers` from make_layers()."""
-    lib = load()
-    f32, i8, u8 = torch.float32, torch.int8, torch.uint8
-    rc = lib.kf_kalman_chain(ctypes.byref(params), layout, _ptr(state, "state", f32),
-                             _ptr(cov, "cov", f32), _ptr(charge, "charge", i8),
-                             _ptr(hits, "hits", f32), _ptr(hit_covs, "hit_covs", f32),
-                             layers, len(layers), _ptr(status, "status", u8), _stream(stream))
-    _check(rc)
+    rc = (_lib or load()).kf_kalman_chain(
+        ctypes.byref(params), layout, _dptr(state, "state", _F32), _dptr(cov, "cov", _F32),
+        _dptr(charge, "charge", _I8), _dptr(hits, "hits", _F32),
+        _dptr(hit_covs, "hit_covs", _F32), layers, len(layers), _dptr(status, "status", _U8),
+        _stream(stream))
+    if rc != KF_OK:
+        _check(rc)
 
 
 def kf_propagate_update_compressed(kind, params, layout, state_in, sigma_in, rho_in, state_out,
                                    sigma_out, rho_out, charge, hit, hit_cov, surf,
                                    surf_per_track=0, status=None, stream=None):
     """C-ABI kf_propagate_update_compressed; rho tensors hold float16 (or int16 bits)."""
-    lib = load()
-    f32, i8, u8 = torch.float32, torch.int8, torch.uint8
-    rc = lib.kf_propagate_update_compressed(
-        int(kind), ctypes.byref(params), layout, _ptr(state_in, "state_in", f32),
-        _ptr(sigma_in, "sigma_in", f32), _ptr(rho_in, "rho_in", torch.float16),
-        _ptr(state_out, "state_out", f32), _ptr(sigma_out, "sigma_out", f32),
-        _ptr(rho_out, "rho_out", torch.float16), _ptr(charge, "charge", i8),
-        _ptr(hit, "hit", f32), _ptr(hit_cov, "hit_cov", f32), _ptr(surf, "surf", f32),
-        int(surf_per_track), _ptr(status, "status", u8), _stream(stream))
-    _check(rc)
+    rc = (_lib or load()).kf_propagate_update_compressed(
+        int(kind), ctypes.byref(params), layout, _dptr(state_in, "state_in", _F32),
+        _dptr(sigma_in, "sigma_in", _F32), _dptr(rho_in, "rho_in", _F16),
+        _dptr(state_out, "state_out", _F32), _dptr(sigma_out, "sigma_out", _F32),
+        _dptr(rho_out, "rho_out", _F16), _dptr(charge, "charge", _I8),
+        _dptr(hit, "hit", _F32), _dptr(hit_cov, "hit_cov", _F32), _dptr(surf, "surf", _F32),
+        int(surf_per_track), _dptr(status, "status", _U8), _stream(stream))
+    if rc != KF_OK:
+        _check(rc)
 
 
 def to_device_rho(rho: np.ndarray, layout: kf_layout, device) -> torch.Tensor:
