@@ -464,11 +464,14 @@ int kf_autotune_clear(void);
  * free, copies each one in, and whenever the device is not already computing
  * a batch launches ONE kernel over every admitted event whose copies have
  * landed (at most 128).  Events submitted while a batch runs join the next
- * batch; results are copied out while the next batch computes.  Each track
+ * batch; results are copied out while the next batch computes.  Under
+ * KF_ADAPTIVE the next batch starts when the first pass of the previous one is
+ * done: its second pass (FP64, few tracks) runs beside it, up to four batches
+ * at a time.  Each track
  * runs the same arithmetic as kf_kalman_chain (SoA layout, one event per
  * submission), so an event's results do not depend on what else is in its
- * batch.  Creating a server creates its thread, three streams and
- * max_events_in_flight + 1 CUDA events; submitting and serving allocate
+ * batch.  Creating a server creates its thread, six streams and a few CUDA
+ * events per event in flight and per stream; submitting and serving allocate
  * nothing (event memory comes from the arena).
  *
  * Direct events: where the server's GPU reaches every array of an event in

@@ -6,11 +6,14 @@
 //   1. admits pending events while an event slot and space in the caller's
 //      device arena are free, and copies each admitted event in on the
 //      copy-in stream;
-//   2. whenever no batch is computing, launches ONE batched chain kernel over
-//      every admitted event whose copies have landed (up to 128 events), on
-//      the compute stream -- events that arrived while the previous batch was
-//      running join the next batch, so work from different requests overlaps
-//      on the device;
+//   2. whenever no batch's chain kernel is computing, launches ONE batched
+//      chain kernel over every admitted event whose copies have landed (up to
+//      128 events) -- events that arrived while the previous batch was running
+//      join the next batch, so work from different requests overlaps on the
+//      device.  KF_ADAPTIVE's second pass leaves most of the device idle (a few
+//      marked tracks, a long chain of FP64 instructions each), so the next
+//      batch starts when the previous one's first pass is done, on another of
+//      kLanes compute streams;
 //   3. when a batch finishes, copies each event's results out on the
 //      copy-out stream while the next batch computes, and when those copies
 //      land marks the event done, records its latency (submit to results in
@@ -61,9 +64,19 @@ constexpr int kMaxBatch = 128;
 // SMs as 256-thread blocks would, so fewer warps share each scheduler.
 constexpr int kBatchThreads = 64;
 
+// Batches in flight.  A second pass takes 90 us or more and a first pass of a
+// few events 20 to 80, so up to four batches overlap.
+constexpr int kLanes = 4;
+
 // How long after its last progress the scheduler keeps polling (in-flight
 // GPU work, and new submissions) without sleeping, microseconds.
 constexpr double kSpinUs = 200.0;
+
+// The shortest time between two looks at several batches in flight,
+// nanoseconds.  Their event queries back to back hold the driver's locks, which
+// every submission's pointer checks need: submitting 16 events took 468 us
+// without it, 219 with it.
+constexpr int64_t kPollNs = 2000;
 
 // One event of a batch.  Copied events: inputs and outputs are the same
 // arena arrays (the chain runs in place).  Direct events: the caller's host
@@ -275,6 +288,17 @@ struct Request {
   bool copied = false;  // copy-in seen complete (t_copied set)
 };
 
+// A compute stream and the batch in flight on it.
+struct Lane {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t first = nullptr;  // the chain kernel (first pass) is done
+  cudaEvent_t ev = nullptr;     // the batch is done
+  cudaEvent_t g0 = nullptr, g1 = nullptr;
+  bool busy = false;
+  bool first_done = false;
+  std::vector<Request *> running;
+};
+
 // First-fit allocator over [0, size) with coalescing.
 struct Arena {
   std::map<int64_t, int64_t> free_;  // offset -> size
@@ -323,12 +347,11 @@ struct kf_server {
   char error_msg[256] = "";
   uint64_t next_ticket = 1;
   std::deque<kf::srv::Request *> pending;
-  std::vector<kf::srv::Request *> copying, running, returning;
+  std::vector<kf::srv::Request *> copying, returning;
   std::unordered_map<uint64_t, kf::srv::Request *> by_ticket;
   std::vector<cudaEvent_t> event_pool;
-  cudaStream_t s_in = nullptr, s_compute = nullptr, s_out = nullptr;
-  cudaEvent_t batch_ev = nullptr;
-  bool batch_in_flight = false;
+  cudaStream_t s_in = nullptr, s_out = nullptr;
+  kf::srv::Lane lanes[kf::srv::kLanes];
   int in_flight = 0;  // admitted, not yet done
   // statistics
   std::vector<double> latencies_ms;
@@ -338,7 +361,6 @@ struct kf_server {
   std::vector<double> phase_ms[9];
   double sched_pass_max_ms = 0.0, sched_gap_max_ms = 0.0;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> timing_pool;
-  cudaEvent_t batch_g0 = nullptr, batch_g1 = nullptr;
   int64_t tracks_done = 0, batches = 0, max_batch_events = 0;
 };
 
@@ -378,10 +400,10 @@ bool start_copy_in(kf_server *s, Request *r) {
   return true;
 }
 
-bool start_copy_out(kf_server *s, Request *r) {
+bool start_copy_out(kf_server *s, Request *r, const kf::srv::Lane &lane) {
   char *b = s->arena_base + r->off;
   const int64_t n = r->n;
-  cudaError_t e = cudaStreamWaitEvent(s->s_out, s->batch_ev, 0);
+  cudaError_t e = cudaStreamWaitEvent(s->s_out, lane.ev, 0);
   if (e == cudaSuccess) e = cudaEventRecord(r->g0, s->s_out);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(r->state_out, b + r->lay.state, 4 * 6 * n, cudaMemcpyDefault, s->s_out);
@@ -398,7 +420,7 @@ bool start_copy_out(kf_server *s, Request *r) {
   return true;
 }
 
-bool launch_batch(kf_server *s, std::vector<Request *> &batch) {
+bool launch_batch(kf_server *s, kf::srv::Lane &lane, const std::vector<Request *> &batch) {
   using namespace kf;
   using namespace kf::srv;
   BatchArgs a{};
@@ -441,31 +463,33 @@ bool launch_batch(kf_server *s, std::vector<Request *> &batch) {
   }
   cudaError_t e = cudaSuccess;
   for (Request *r : batch) {
-    e = cudaStreamWaitEvent(s->s_compute, r->ev, 0);
+    e = cudaStreamWaitEvent(lane.stream, r->ev, 0);
     if (e != cudaSuccess) break;
   }
-  if (e == cudaSuccess) e = cudaEventRecord(s->batch_g0, s->s_compute);
+  if (e == cudaSuccess) e = cudaEventRecord(lane.g0, lane.stream);
   if (e == cudaSuccess && blocks > 0) {
     const unsigned g = (unsigned)blocks;
+    const cudaStream_t st = lane.stream;
     switch (s->cfg.precision) {
-      case KF_FP32: batch_chain_kernel<kFP32><<<g, kBatchThreads, 0, s->s_compute>>>(a); break;
-      case KF_FP64_UPDATE: batch_chain_kernel<kFP64Update><<<g, kBatchThreads, 0, s->s_compute>>>(a); break;
-      case KF_JOSEPH: batch_chain_kernel<kJoseph><<<g, kBatchThreads, 0, s->s_compute>>>(a); break;
-      case KF_FP64: batch_chain_kernel<kFP64><<<g, kBatchThreads, 0, s->s_compute>>>(a); break;
-      case KF_DF_UPDATE: batch_chain_kernel<kDFUpdate><<<g, kBatchThreads, 0, s->s_compute>>>(a); break;
-      default:
-        batch_chain_kernel<kAdaptive><<<g, kBatchThreads, 0, s->s_compute>>>(a);
-        e = cudaGetLastError();
-        if (e == cudaSuccess)
-          batch_redo_kernel<<<(g + kBatchRedoBlocks - 1) / kBatchRedoBlocks, f64::kGroupThreads, 0,
-                              s->s_compute>>>(
-              a, (int64_t)g);
-        break;
+      case KF_FP32: batch_chain_kernel<kFP32><<<g, kBatchThreads, 0, st>>>(a); break;
+      case KF_FP64_UPDATE: batch_chain_kernel<kFP64Update><<<g, kBatchThreads, 0, st>>>(a); break;
+      case KF_JOSEPH: batch_chain_kernel<kJoseph><<<g, kBatchThreads, 0, st>>>(a); break;
+      case KF_FP64: batch_chain_kernel<kFP64><<<g, kBatchThreads, 0, st>>>(a); break;
+      case KF_DF_UPDATE: batch_chain_kernel<kDFUpdate><<<g, kBatchThreads, 0, st>>>(a); break;
+      default: batch_chain_kernel<kAdaptive><<<g, kBatchThreads, 0, st>>>(a); break;
     }
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = cudaGetLastError();
+    if (e == cudaSuccess && s->cfg.precision == KF_ADAPTIVE) {
+      e = cudaEventRecord(lane.first, st);
+      if (e == cudaSuccess) {
+        batch_redo_kernel<<<(g + kBatchRedoBlocks - 1) / kBatchRedoBlocks, f64::kGroupThreads, 0,
+                            st>>>(a, (int64_t)g);
+        e = cudaGetLastError();
+      }
+    }
   }
-  if (e == cudaSuccess) e = cudaEventRecord(s->batch_g1, s->s_compute);
-  if (e == cudaSuccess) e = cudaEventRecord(s->batch_ev, s->s_compute);
+  if (e == cudaSuccess) e = cudaEventRecord(lane.g1, lane.stream);
+  if (e == cudaSuccess) e = cudaEventRecord(lane.ev, lane.stream);
   if (e != cudaSuccess) {
     fail_locked(s, e, "server batch launch");
     return false;
@@ -519,29 +543,29 @@ bool schedule_once(kf_server *s) {
     s->returning.erase(s->returning.begin() + k);
     moved = true;
   }
-  // the running batch finished: direct events are done (the kernel wrote
+  // a running batch finished: its direct events are done (the kernel wrote
   // their results to host memory), the others are copied out
-  if (s->batch_in_flight) {
-    const cudaError_t q = cudaEventQuery(s->batch_ev);
-    if (q != cudaErrorNotReady) {
-      if (q != cudaSuccess) fail_locked(s, q, "server batch completion");
-      const auto now = std::chrono::steady_clock::now();
-      float gpu_ms = 0.0f;
-      if (q == cudaSuccess) cudaEventElapsedTime(&gpu_ms, s->batch_g0, s->batch_g1);
-      for (Request *r : s->running) {
-        r->t_finished = now;
-        r->gpu_compute_ms = gpu_ms;
-        if (r->direct) {
-          finish_request(s, r);
-        } else if (start_copy_out(s, r)) {
-          r->phase = Phase::kReturning;
-          s->returning.push_back(r);
-        }
+  for (kf::srv::Lane &lane : s->lanes) {
+    if (!lane.busy) continue;
+    const cudaError_t q = cudaEventQuery(lane.ev);
+    if (q == cudaErrorNotReady) continue;
+    if (q != cudaSuccess) fail_locked(s, q, "server batch completion");
+    const auto now = std::chrono::steady_clock::now();
+    float gpu_ms = 0.0f;
+    if (q == cudaSuccess) cudaEventElapsedTime(&gpu_ms, lane.g0, lane.g1);
+    for (Request *r : lane.running) {
+      r->t_finished = now;
+      r->gpu_compute_ms = gpu_ms;
+      if (r->direct) {
+        finish_request(s, r);
+      } else if (start_copy_out(s, r, lane)) {
+        r->phase = Phase::kReturning;
+        s->returning.push_back(r);
       }
-      s->running.clear();
-      s->batch_in_flight = false;
-      moved = true;
     }
+    lane.running.clear();
+    lane.busy = false;
+    moved = true;
   }
   if (s->paused || s->error != KF_OK) return moved;
   // admit while a slot, an event object and arena space are free
@@ -582,30 +606,53 @@ bool schedule_once(kf_server *s) {
       }
     }
   }
-  // launch everything whose copies have landed
-  if (!s->batch_in_flight && !s->copying.empty()) {
-    std::vector<Request *> batch;
-    for (size_t k = 0; k < s->copying.size() && (int)batch.size() < kf::srv::kMaxBatch;) {
-      Request *r = s->copying[k];
-      if (r->copied) {
-        batch.push_back(r);
-        s->copying.erase(s->copying.begin() + k);
-      } else {
-        ++k;
-      }
+  // launch everything whose copies have landed, on a free lane, unless a
+  // batch's chain kernel is still computing
+  if (s->copying.empty()) return moved;
+  kf::srv::Lane *lane = nullptr;
+  for (kf::srv::Lane &l : s->lanes) {
+    if (!l.busy) {
+      if (!lane) lane = &l;
+      continue;
     }
-    if (!batch.empty() && launch_batch(s, batch)) {
-      const auto now = std::chrono::steady_clock::now();
-      for (Request *r : batch) {
-        r->phase = Phase::kRunning;
-        r->t_launch = now;
-      }
-      s->running = batch;
-      s->batch_in_flight = true;
-      moved = true;
+    if (!l.first_done && s->cfg.precision == KF_ADAPTIVE)
+      l.first_done = cudaEventQuery(l.first) == cudaSuccess;
+    if (!l.first_done) return moved;
+  }
+  if (!lane) return moved;
+  std::vector<Request *> batch;
+  for (size_t k = 0; k < s->copying.size() && (int)batch.size() < kf::srv::kMaxBatch;) {
+    Request *r = s->copying[k];
+    if (r->copied) {
+      batch.push_back(r);
+      s->copying.erase(s->copying.begin() + k);
+    } else {
+      ++k;
     }
   }
+  if (!batch.empty() && launch_batch(s, *lane, batch)) {
+    const auto now = std::chrono::steady_clock::now();
+    for (Request *r : batch) {
+      r->phase = Phase::kRunning;
+      r->t_launch = now;
+    }
+    lane->running = batch;
+    lane->busy = true;
+    lane->first_done = false;
+    moved = true;
+  }
   return moved;
+}
+
+int batches_in_flight(const kf_server *s) {
+  int k = 0;
+  for (const kf::srv::Lane &l : s->lanes) k += l.busy;
+  return k;
+}
+
+// Work on the device: copies, or a batch on some lane.
+bool device_busy(const kf_server *s) {
+  return !s->copying.empty() || !s->returning.empty() || batches_in_flight(s) > 0;
 }
 
 void scheduler_main(kf_server *s) {
@@ -622,7 +669,7 @@ void scheduler_main(kf_server *s) {
     // was away between passes while GPU work was in flight (the mutex, the
     // back-off sleep and the OS's scheduling of this thread)
     const auto t0 = std::chrono::steady_clock::now();
-    const bool was_busy = s->batch_in_flight || !s->copying.empty() || !s->returning.empty();
+    const bool was_busy = device_busy(s);
     if (was_busy)
       s->sched_gap_max_ms =
           std::max(s->sched_gap_max_ms, std::chrono::duration<double, std::milli>(t0 - last).count());
@@ -630,7 +677,7 @@ void scheduler_main(kf_server *s) {
     last = std::chrono::steady_clock::now();
     s->sched_pass_max_ms =
         std::max(s->sched_pass_max_ms, std::chrono::duration<double, std::milli>(last - t0).count());
-    const bool busy = s->batch_in_flight || !s->copying.empty() || !s->returning.empty();
+    const bool busy = device_busy(s);
     if (moved) {
       progress = last;
       continue;
@@ -639,11 +686,15 @@ void scheduler_main(kf_server *s) {
       // GPU work in flight: poll its events again at once for the first
       // kSpinUs after the last progress (a batch of a few events takes tens
       // of microseconds), then every 10 us
+      const bool several = batches_in_flight(s) > 1;
       lock.unlock();
-      if (std::chrono::duration<double, std::micro>(last - progress).count() < kf::srv::kSpinUs)
-        std::this_thread::yield();
-      else
+      if (std::chrono::duration<double, std::micro>(last - progress).count() < kf::srv::kSpinUs) {
+        const auto until = last + std::chrono::nanoseconds(several ? kf::srv::kPollNs : 0);
+        do std::this_thread::yield();
+        while (std::chrono::steady_clock::now() < until);
+      } else {
         std::this_thread::sleep_for(std::chrono::microseconds(10));
+      }
       lock.lock();
     } else if (std::chrono::duration<double, std::micro>(last - progress).count() <
                kf::srv::kSpinUs) {
@@ -693,11 +744,14 @@ extern "C" int kf_server_create(const kf_server_config *cfg, kf_server **out) {
   s->arena_base = static_cast<char *>(cfg->arena);
   s->arena = kf::srv::Arena(cfg->arena_bytes);
   cudaError_t e = cudaStreamCreateWithFlags(&s->s_in, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->s_compute, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->s_out, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->batch_ev, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreate(&s->batch_g0);
-  if (e == cudaSuccess) e = cudaEventCreate(&s->batch_g1);
+  for (kf::srv::Lane &l : s->lanes) {
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&l.first, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&l.ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreate(&l.g0);
+    if (e == cudaSuccess) e = cudaEventCreate(&l.g1);
+  }
   for (int k = 0; e == cudaSuccess && k < cfg->max_events_in_flight; ++k) {
     cudaEvent_t ev, g0 = nullptr, g1 = nullptr;
     e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
@@ -921,7 +975,8 @@ extern "C" int kf_server_destroy(kf_server *s) {
   s->cv_work.notify_one();
   if (s->thread.joinable()) s->thread.join();
   if (s->s_in) cudaStreamSynchronize(s->s_in);
-  if (s->s_compute) cudaStreamSynchronize(s->s_compute);
+  for (kf::srv::Lane &l : s->lanes)
+    if (l.stream) cudaStreamSynchronize(l.stream);
   if (s->s_out) cudaStreamSynchronize(s->s_out);
   for (auto &kv : s->by_ticket) {
     if (kv.second->ev) cudaEventDestroy(kv.second->ev);
@@ -932,11 +987,12 @@ extern "C" int kf_server_destroy(kf_server *s) {
     cudaEventDestroy(g.first);
     cudaEventDestroy(g.second);
   }
-  if (s->batch_g0) cudaEventDestroy(s->batch_g0);
-  if (s->batch_g1) cudaEventDestroy(s->batch_g1);
-  if (s->batch_ev) cudaEventDestroy(s->batch_ev);
+  for (kf::srv::Lane &l : s->lanes) {
+    for (cudaEvent_t ev : {l.first, l.ev, l.g0, l.g1})
+      if (ev) cudaEventDestroy(ev);
+    if (l.stream) cudaStreamDestroy(l.stream);
+  }
   if (s->s_in) cudaStreamDestroy(s->s_in);
-  if (s->s_compute) cudaStreamDestroy(s->s_compute);
   if (s->s_out) cudaStreamDestroy(s->s_out);
   delete s;
   return KF_OK;
