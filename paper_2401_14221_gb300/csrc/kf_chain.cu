@@ -64,26 +64,9 @@ __device__ __forceinline__ void chain_redo_group(const ChainArgs &a, const f64::
   if (g.role == 0 && store && a.status) a.status[i] = (uint8_t)st;
 }
 
-// The second pass over one list of the whole batch's marked tracks.
-// chain_compact_kernel builds the list: each block gathers its span's marks
-// and appends them (one atomic per block; the order of the list varies from
-// run to run, the result of each track does not).
-__global__ void __launch_bounds__(f64::kGroupThreads) chain_compact_kernel(const uint8_t *status,
-                                                                     int64_t n,
-                                                                     uint32_t *count,
-                                                                     uint32_t *list) {
-  __shared__ uint16_t span_list[kChainSpan];
-  __shared__ int span_count;
-  __shared__ uint32_t base;
-  const int64_t span0 = (int64_t)blockIdx.x * kChainSpan;
-  const int cnt = gather_marked<kChainSpan, f64::kGroupThreads>(status, span0, n, span_list, &span_count);
-  if (cnt == 0) return;  // the same count in every thread of the block
-  if (threadIdx.x == 0) base = atomicAdd(count, (uint32_t)cnt);
-  __syncthreads();
-  for (int q = threadIdx.x; q < cnt; q += blockDim.x)
-    list[base + q] = (uint32_t)(span0 + span_list[q]);
-}
-
+// The second pass over one list of the whole batch's marked tracks, which the
+// first pass appends to (an atomic per marked track; the order of the list
+// varies from run to run, the result of each track does not).
 constexpr int kRedoListBlocksPerSm = 4;
 // Up to this many tracks per SM four warps share 32 tracks, beyond it each
 // thread runs a track.  KF_FP64 chain of 15 layers, us: one group per SM (up
@@ -92,9 +75,12 @@ constexpr int kRedoListBlocksPerSm = 4;
 constexpr int kGroupTracksPerSm = 96;
 
 __global__ void __launch_bounds__(f64::kGroupThreads, kRedoListBlocksPerSm)
-    chain_redo_list_kernel(const ChainArgs a, const uint32_t *count, const uint32_t *list) {
+    chain_redo_list_kernel(const __grid_constant__ ChainArgs a) {
   __shared__ f64::Shared sh;
-  const int64_t total = *count;
+  // the marking pass's list, complete once that kernel is
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t total = *a.redo_count;
+  const uint32_t *list = a.redo_list;
   if (total > (int64_t)(gridDim.x / kRedoListBlocksPerSm) * kGroupTracksPerSm) {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
          q += (int64_t)gridDim.x * blockDim.x)
@@ -168,38 +154,57 @@ bool redo_pool(int dev, bool may_create, cudaMemPool_t *out) {
 
 std::atomic<int> g_chain_redo{KF_CHAIN_REDO_LIST};
 
-// Launch the second pass on stream s: over a compacted list when its
-// scratch can be allocated, else per span (the same results).
-int launch_chain_redo(const ChainArgs &a, cudaStream_t s) {
-  const unsigned spans = (unsigned)((a.n + kChainSpan - 1) / kChainSpan);
-  int dev = 0, sms = 0;
+// Give the first pass a list for the tracks it marks, its count zeroed on
+// stream s: stream-ordered scratch, to be returned with cudaFreeAsync.  False
+// (and no list) when the marks alone have to do.
+bool start_redo_list(ChainArgs &a, int dev, cudaStream_t s) {
   cudaMemPool_t pool = nullptr;
   void *buf = nullptr;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   const bool capturing = cudaStreamIsCapturing(s, &capture) != cudaSuccess ||
                          capture != cudaStreamCaptureStatusNone;
   if (g_chain_redo.load(std::memory_order_relaxed) == KF_CHAIN_REDO_LIST &&
-      a.n < (int64_t)UINT32_MAX && cudaGetDevice(&dev) == cudaSuccess &&
-      staged::sm_count(dev, &sms) == KF_OK && redo_pool(dev, !capturing, &pool) &&
+      a.n < (int64_t)UINT32_MAX && redo_pool(dev, !capturing, &pool) &&
       cudaMallocFromPoolAsync(&buf, 4 * (size_t)(a.n + 1), pool, s) == cudaSuccess) {
-    uint32_t *count = static_cast<uint32_t *>(buf), *list = count + 1;
-    int rc = check_cuda(cudaMemsetAsync(count, 0, sizeof(uint32_t), s), "cudaMemsetAsync");
-    if (rc == KF_OK) {
-      chain_compact_kernel<<<spans, f64::kGroupThreads, 0, s>>>(a.status, a.n, count, list);
-      rc = check_cuda(cudaGetLastError(), "chain compaction launch");
+    if (cudaMemsetAsync(buf, 0, sizeof(uint32_t), s) == cudaSuccess) {
+      a.redo_count = static_cast<uint32_t *>(buf);
+      a.redo_list = a.redo_count + 1;
+      return true;
     }
-    if (rc == KF_OK) {
-      chain_redo_list_kernel<<<(unsigned)(kRedoListBlocksPerSm * sms), f64::kGroupThreads, 0, s>>>(
-          a, count, list);
+    (void)cudaFreeAsync(buf, s);
+  }
+  (void)cudaGetLastError();  // a refused allocation is not the caller's error
+  return false;
+}
+
+// KF_ADAPTIVE: the marking pass, then the second pass over its list, or per
+// span where there is none (the same results).
+int launch_chain_adaptive(ChainArgs &a, unsigned blocks, int threads, int dev, int sms,
+                          cudaStream_t s) {
+  const bool list = start_redo_list(a, dev, s);
+  int rc = launch_chain_mark(a, blocks, threads, s);
+  if (rc == KF_OK) {
+    if (list) {
+      // a programmatic dependent: set up while the marking pass drains
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(kRedoListBlocksPerSm * sms));
+      cfg.blockDim = dim3(f64::kGroupThreads);
+      cfg.stream = s;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      rc = check_cuda(cudaLaunchKernelEx(&cfg, chain_redo_list_kernel, a), "chain redo pass launch");
+    } else {
+      chain_redo_kernel<<<(unsigned)((a.n + kChainSpan - 1) / kChainSpan), f64::kGroupThreads, 0,
+                          s>>>(a);
       rc = check_cuda(cudaGetLastError(), "chain redo pass launch");
     }
-    const cudaError_t freed = cudaFreeAsync(buf, s);  // returned to the pool on every path
-    return rc != KF_OK ? rc : check_cuda(freed, "cudaFreeAsync");
   }
-  clear_error();
-  (void)cudaGetLastError();  // a refused allocation is not the caller's error
-  chain_redo_kernel<<<spans, f64::kGroupThreads, 0, s>>>(a);
-  return check_cuda(cudaGetLastError(), "chain redo pass launch");
+  if (!list) return rc;
+  const cudaError_t freed = cudaFreeAsync(a.redo_count, s);  // returned on every path
+  return rc != KF_OK ? rc : check_cuda(freed, "cudaFreeAsync");
 }
 
 }  // namespace
@@ -293,14 +298,12 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   int rc = KF_OK;
   switch (params->precision) {
     case KF_FP32: rc = launch_chain_fp32(a, g, threads, s); break;
-    case KF_ADAPTIVE: rc = launch_chain_mark(a, g, threads, s); break;
+    case KF_ADAPTIVE: return launch_chain_adaptive(a, g, threads, dev, sms, s);
     case KF_FP64_UPDATE: chain_kernel<kFP64Update, 0><<<g, threads, 0, s>>>(a); break;
     case KF_JOSEPH: rc = launch_chain_joseph(a, g, threads, s); break;
     case KF_FP64: chain_kernel<kFP64, 0><<<g, threads, 0, s>>>(a); break;
-    default: chain_kernel<kDFUpdate, 0><<<g, threads, 0, s>>>(a); break;
+    default: rc = launch_chain_df(a, g, threads, s); break;
   }
   if (rc != KF_OK) return rc;
-  if (int rc2 = check_cuda(cudaGetLastError(), "chain launch")) return rc2;
-  if (params->precision != KF_ADAPTIVE) return KF_OK;
-  return launch_chain_redo(a, s);
+  return check_cuda(cudaGetLastError(), "chain launch");
 }

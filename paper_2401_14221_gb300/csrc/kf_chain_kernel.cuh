@@ -25,6 +25,10 @@ struct ChainArgs {
   int32_t L;
   int32_t kinds[KF_MAX_LAYERS];
   float pos[KF_MAX_LAYERS];
+  // where KF_ADAPTIVE's first pass lists the tracks it marks (NULL: status
+  // marks only)
+  uint32_t *redo_count = nullptr;
+  uint32_t *redo_list = nullptr;
 };
 
 // Track i of the chain: load, run every layer, store.
@@ -48,8 +52,9 @@ __device__ __forceinline__ void chain_one(const ChainArgs &a, int64_t i) {
   if constexpr (VARIANT == kAdaptive) {
     st = chain_track_marking(p, C, qf, a.bz, a.L, a.kinds, a.pos, a.hits, a.hit_stride, a.hitcovs,
                              a.hc_stride, l3, l6);
-    if (st & kRedo) {  // left to chain_redo_kernel, inputs untouched
+    if (st & kRedo) {  // left to the second pass, inputs untouched
       a.status[i] = (uint8_t)kRedo;
+      if (a.redo_list) a.redo_list[atomicAdd(a.redo_count, 1u)] = (uint32_t)i;
       return;
     }
   } else if constexpr (VARIANT == kFP64) {
@@ -82,23 +87,27 @@ __global__ void __launch_bounds__(256, VARIANT == kAdaptive ? 3 : 0)
 // The kernel with the AoSoA width known at compile time: a hit's nine loads
 // then differ by immediate offsets, which takes 4 % of the chain's instructions
 // and the 64-bit strides out of its registers (1.75 M tracks, FP32 391 -> 381
-// us, Joseph 467 -> 455, adaptive 605 -> 586).
+// us, Joseph 467 -> 455, double-float update 838 -> 817, adaptive 605 -> 586).
+// SoA gets a kernel too, but for the double-float update, whose SoA kernel
+// spills (860 us; 838 with strides known at run time).
 template <int VARIANT>
 int launch_chain_by_width(const ChainArgs &a, unsigned blocks, int threads, cudaStream_t s) {
+  constexpr int kSoa = VARIANT == kDFUpdate ? 0 : -1;
   switch (a.soa ? -1 : a.lw) {
     case 4: chain_kernel<VARIANT, 4><<<blocks, threads, 0, s>>>(a); break;
     case 5: chain_kernel<VARIANT, 5><<<blocks, threads, 0, s>>>(a); break;
     case 6: chain_kernel<VARIANT, 6><<<blocks, threads, 0, s>>>(a); break;
     case 7: chain_kernel<VARIANT, 7><<<blocks, threads, 0, s>>>(a); break;
-    default: chain_kernel<VARIANT, -1><<<blocks, threads, 0, s>>>(a); break;
+    default: chain_kernel<VARIANT, kSoa><<<blocks, threads, 0, s>>>(a); break;
   }
   return check_cuda(cudaGetLastError(), "chain launch");
 }
 
 // Instantiated in units of their own (kf_chain_fp32.cu, kf_chain_joseph.cu,
-// kf_chain_mark.cu).
+// kf_chain_df.cu, kf_chain_mark.cu).
 int launch_chain_fp32(const ChainArgs &a, unsigned blocks, int threads, cudaStream_t s);
 int launch_chain_joseph(const ChainArgs &a, unsigned blocks, int threads, cudaStream_t s);
+int launch_chain_df(const ChainArgs &a, unsigned blocks, int threads, cudaStream_t s);
 int launch_chain_mark(const ChainArgs &a, unsigned blocks, int threads, cudaStream_t s);
 
 }  // namespace kf
