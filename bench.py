@@ -150,7 +150,8 @@ def profiled_traffic(shape):
 CHAIN_SOURCES = ("paper_2401_14221_gb300/csrc/kf_num.cuh",
                  "paper_2401_14221_gb300/csrc/kf_device.cuh",
                  "paper_2401_14221_gb300/csrc/kf_chain.cuh",
-                 "paper_2401_14221_gb300/csrc/kf_chain.cu",
+                 "paper_2401_14221_gb300/csrc/kf_chain_kernel.cuh",
+                 "paper_2401_14221_gb300/csrc/kf_chain_fp32.cu",
                  "paper_2401_14221_gb300/build.py")
 
 

@@ -73,12 +73,10 @@ __device__ __forceinline__ void chain_one(const ChainArgs &a, int64_t i) {
 }
 
 // One track per thread.  KF_ADAPTIVE's first pass is the same kernel (kAdaptive:
-// marked tracks are left alone), held to 80 registers so that three 256-thread
-// CTAs fit an SM (unbounded it takes 96: the 256-event chain 1.057 against
-// 0.949 ms; 72 and 64 registers spill and lose 1 to 6 %).  The other float
-// variants take 80 by themselves.
+// marked tracks are left alone).  The float variants take 80 registers: 72 and
+// 64 spill and lose 1 to 6 %, 88 gain nothing.
 template <int VARIANT, int LW>
-__global__ void __launch_bounds__(256, VARIANT == kAdaptive ? 3 : 0)
+__global__ void __launch_bounds__(256)
     chain_kernel(const __grid_constant__ ChainArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < a.n) chain_one<VARIANT, LW>(a, i);
@@ -87,7 +85,7 @@ __global__ void __launch_bounds__(256, VARIANT == kAdaptive ? 3 : 0)
 // The kernel with the AoSoA width known at compile time: a hit's nine loads
 // then differ by immediate offsets, which takes 4 % of the chain's instructions
 // and the 64-bit strides out of its registers (1.75 M tracks, FP32 391 -> 381
-// us, Joseph 467 -> 455, double-float update 838 -> 817, adaptive 605 -> 586).
+// us, Joseph 467 -> 455, double-float update 838 -> 817, adaptive 605 -> 582).
 // SoA gets a kernel too, but for the double-float update, whose SoA kernel
 // spills (860 us; 838 with strides known at run time).
 template <int VARIANT>
