@@ -55,6 +55,7 @@ NOMINAL_HBM_GBS = 7900.0
 # in profiles/ is valid while these are unchanged)
 KERNEL_SOURCES = ("paper_2401_14221_gb300/csrc/kf_common.cuh",
                   "paper_2401_14221_gb300/csrc/kf_num.cuh",
+                  "paper_2401_14221_gb300/csrc/kf_fp64.cuh",
                   "paper_2401_14221_gb300/csrc/kf_device.cuh",
                   "paper_2401_14221_gb300/csrc/kf_step.cuh",
                   "paper_2401_14221_gb300/csrc/kf_step.cu",

@@ -614,10 +614,12 @@ int kf_set_staged_ctas_per_sm(int32_t ctas);
  * kf_set_chain_redo -- how kf_kalman_chain's KF_ADAPTIVE second pass runs
  * the marked tracks, for all later calls in this process (results are the
  * same, bit for bit):
- *   KF_CHAIN_REDO_LIST  (default) the whole batch's marked tracks in one
- *                       compacted list, 32 to a warp (device scratch from
- *                       the library's pool; per span when it cannot be had)
- *   KF_CHAIN_REDO_SPAN  each 4,096-track span's marked tracks by one block
+ *   KF_CHAIN_REDO_LIST  (default) the whole batch's marked tracks from one
+ *                       list that the first pass writes, 32 at a time by
+ *                       four warps or one to a thread where there are many
+ *                       (device scratch from the library's pool; per span
+ *                       when it cannot be had)
+ *   KF_CHAIN_REDO_SPAN  each 2,048-track span's marked tracks by one block
  * Returns KF_ERR_ARG for any other value.
  */
 #define KF_CHAIN_REDO_LIST 0
