@@ -68,11 +68,17 @@ __device__ __forceinline__ void chain_redo_group(const ChainArgs &a, const f64::
 // first pass appends to (an atomic per marked track; the order of the list
 // varies from run to run, the result of each track does not).
 constexpr int kRedoListBlocksPerSm = 4;
-// Up to this many tracks per SM four warps share 32 tracks, beyond it each
-// thread runs a track.  KF_FP64 chain of 15 layers, us: one group per SM (up
-// to 4,864 tracks) 91, two 122, three 167, four 214; one thread per track 163
-// up to 10,000 tracks, 175 up to 19,000.
+// Up to this many tracks per SM four warps share 32 tracks of a KF_FP64 chain,
+// beyond it each thread runs a track (chain_kernel).  15 layers, us: one group
+// per SM (up to 4,864 tracks) 91, two 122, three 167, four 214; one thread per
+// track 163 up to 10,000 tracks, 175 up to 19,000.
 constexpr int kGroupTracksPerSm = 96;
+// The same line for the list, whose kernel has 128 registers where a thread's
+// track wants 150, and whose blocks land where the first pass leaves room.
+// Adaptive chain, four warps against one thread: 2.6 M tracks (17,000 listed)
+// 809 and 916 us, 5 M (33,000) 1,555 and 1,610, 8 M (52,000, 345 per SM) 2,377
+// and 2,434, 9.5 M (62,000, 410 per SM) 2,838 and 2,769, 13 M 3,829 and 3,693.
+constexpr int kListGroupTracksPerSm = 384;
 
 __global__ void __launch_bounds__(f64::kGroupThreads, kRedoListBlocksPerSm)
     chain_redo_list_kernel(const __grid_constant__ ChainArgs a) {
@@ -81,7 +87,7 @@ __global__ void __launch_bounds__(f64::kGroupThreads, kRedoListBlocksPerSm)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int64_t total = *a.redo_count;
   const uint32_t *list = a.redo_list;
-  if (total > (int64_t)(gridDim.x / kRedoListBlocksPerSm) * kGroupTracksPerSm) {
+  if (total > (int64_t)(gridDim.x / kRedoListBlocksPerSm) * kListGroupTracksPerSm) {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
          q += (int64_t)gridDim.x * blockDim.x)
       chain_redo_track(a, list[q]);

@@ -329,3 +329,23 @@ def test_chain_kernels_of_every_layout_agree_bitwise(dev, n, precision):
     for other in got[1:]:
         for a, b in zip(got[0], other):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("per_sm,more", [(32, 0), (96, 1), (128, 1), (384, 0), (384, 1)])
+def test_adaptive_chain_lists_of_any_length(dev, per_sm, more):
+    # hits so precise that the first layer a track reaches marks it: the second
+    # pass lists every track that reaches one, around the lengths at which its
+    # blocks take a second group and at which a thread runs a track; either way
+    # the bits of the all-FP64 chain
+    n = per_sm * torch.cuda.get_device_properties(dev).multi_processor_count + more
+    cw = W.make_chain(events=1, seed=23, sizes=np.array([n]), pool=512)
+    dc = kf.chain_upload(cw, kf.KF_AOSOA, 32, dev)
+    dc.hit_covs.mul_(1e-10)
+    dc.run(kf.KF_ADAPTIVE)
+    torch.cuda.synchronize()
+    ada = dc.download()
+    dc.reset()
+    dc.run(kf.KF_FP64)
+    torch.cuda.synchronize()
+    for x, y in zip(ada, dc.download()):
+        assert np.array_equal(x.view(np.uint8), y.view(np.uint8))
