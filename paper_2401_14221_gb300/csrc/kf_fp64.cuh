@@ -142,8 +142,10 @@ __device__ __forceinline__ double sqrt(double x) {
 // ------------------------------------------------------------- sin and cos
 // sin and cos of k pi/128, k = 0..255, evaluated at compile time by Taylor
 // series in double-double arithmetic (Knuth's two-sum, Dekker's product) and
-// rounded to double.
-struct SinCosTable {
+// rounded to double.  Read as double2 (table_entry), so the table is aligned
+// like one: doubles alone would ask for 8 bytes, and a 16-byte load faults on
+// an address that is no multiple of 16.
+struct alignas(alignof(double2)) SinCosTable {
   double v[256][2];
 };
 
