@@ -58,6 +58,7 @@ KERNEL_SOURCES = ("paper_2401_14221_gb300/csrc/kf_common.cuh",
                   "paper_2401_14221_gb300/csrc/kf_fp64.cuh",
                   "paper_2401_14221_gb300/csrc/kf_device.cuh",
                   "paper_2401_14221_gb300/csrc/kf_step.cuh",
+                  "paper_2401_14221_gb300/csrc/kf_step_kernel.cuh",
                   "paper_2401_14221_gb300/csrc/kf_step.cu",
                   "paper_2401_14221_gb300/csrc/kf_step_staged.cuh",
                   "paper_2401_14221_gb300/csrc/kf_step_staged.cu",

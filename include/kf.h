@@ -130,6 +130,12 @@ typedef struct {
                                (GB300 issues FP64 at 1/64 of FP32).  In the
                                chain the state is rounded to FP32 between
                                layers, as for KF_FP64_UPDATE.                */
+/*
+ * Denormal floats: double arithmetic (KF_FP64 and the redo of KF_ADAPTIVE)
+ * takes and returns them as they are, and so does the whole single step under
+ * KF_FP64_UPDATE, whichever kernel runs it; other FP32 arithmetic flushes them
+ * to zero.
+ */
 
 typedef struct {
     float    bz;        /* field along +z in tesla                          */

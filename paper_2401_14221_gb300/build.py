@@ -23,14 +23,14 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
               "--expt-relaxed-constexpr", f"-I{INCLUDE}", f"-I{CSRC}"]
 # FP32 denormals flush to zero (-ftz=true) in every translation unit except
-# the staged kernel's double-arithmetic instantiations (*_f64.cu).  No
+# those of the single step's double-arithmetic variants (*_f64.cu).  No
 # quantity of the step comes near the denormal range (the smallest are
 # covariance elements of ~1e-16).  Without denormal handling the FP32 sqrt,
 # division and special-function sequences are shorter: the issue-bound chain
 # runs 5-7 % faster, with results on a 64-event workload bit for bit those
-# of the build without the flag.  The FP64 variants run 5-14 % slower with
-# it (more float<->double conversion work), so their staged units keep IEEE
-# denormals.
+# of the build without the flag.  Double arithmetic itself takes and returns
+# denormal floats in every unit (its conversions do not depend on the flag);
+# in the *_f64.cu units the FP32 transport of KF_FP64_UPDATE keeps them too.
 FTZ_FLAGS = ["-ftz=true"]
 
 

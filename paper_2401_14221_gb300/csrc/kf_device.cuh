@@ -485,7 +485,7 @@ __device__ __forceinline__ bool kalman_update_f64(float (&p)[6], float (&C)[21],
   using f64::to_float;
   const double S00 = from_float(S00f), S01 = from_float(S01f), S11 = from_float(S11f);
   const double det = __fma_rn(S00, S11, -__dmul_rn(S01, S01));
-  if (!(S00f > 0.0f) || !f64::gt0(det)) return true;
+  if (!f64::gt0(S00) || !f64::gt0(det)) return true;
   const double inv = f64::rcp(det);
   const double Si00 = __dmul_rn(S11, inv), Si01 = -__dmul_rn(S01, inv), Si11 = __dmul_rn(S00, inv);
   const double V00 = from_float(V00f), V01 = from_float(V01f), V11 = from_float(V11f);

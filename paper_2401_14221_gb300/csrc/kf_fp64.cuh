@@ -45,13 +45,17 @@ __device__ __forceinline__ double from_normal(float f) {
   return __hiloint2double(((i >> 3) & (int)0x8fffffff) + 0x38000000, i << 29);
 }
 
-// (double)f by shifts.  Denormals read as zero (the library is built with
-// -ftz=true); infinities and NaN stay what they are.
+// (double)f by shifts, exact for every float: below the normal range f is
+// scaled up by 2^32 first, by a product that keeps denormals whether or not the
+// unit is built with -ftz=true; infinities and NaN stay what they are.
 __device__ __forceinline__ double from_float(float f) {
-  const int i = __float_as_int(f), e = i & 0x7f800000;
-  const int bias = e == 0x7f800000 ? 0x70000000 : 0x38000000;
+  const int e = __float_as_int(f) & 0x7f800000;
+  float up;
+  asm("mul.rn.f32 %0, %1, 0f4F800000;" : "=f"(up) : "f"(f));
+  const int i = __float_as_int(e == 0 ? up : f);
+  const int bias = e == 0 ? 0x36000000 : e == 0x7f800000 ? 0x70000000 : 0x38000000;
   const int hi = ((i >> 3) & (int)0x8fffffff) + bias;
-  return __hiloint2double(e == 0 ? i & (int)0x80000000 : hi, e == 0 ? 0 : i << 29);
+  return __hiloint2double((i << 1) == 0 ? i : hi, i << 29);
 }
 
 // The high word of |x|: the exponent and 20 bits of the mantissa.
@@ -73,9 +77,14 @@ __device__ __forceinline__ float cut(double x) {
 
 // (float)x, rounded to nearest even: the bits cut off plus just under half a
 // unit (half, if the last bit kept is odd) carry into it.  Zero, and
-// what is not a normal float, take the instruction.
+// what is not a normal float, take the instruction, which keeps denormal
+// results in every unit.
 __device__ __forceinline__ float to_float(double x) {
-  if (top(x) - 0x38100000u >= 0x0fe00000u) return (float)x;
+  if (top(x) - 0x38100000u >= 0x0fe00000u) {
+    float f;
+    asm("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(x));
+    return f;
+  }
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const unsigned m = __funnelshift_l(lo, hi - 0x38000000u, 3) & 0x7fffffffu;
   const unsigned rest = lo << 3;

@@ -109,6 +109,14 @@ struct LaunchConfig {
 int launch_step_kernel(int kind, int precision, const StepArgs &a, cudaStream_t s,
                        bool plain_loads = false);
 
+// Launches of the one-thread-per-track kernels with the double-arithmetic
+// variants (KF_FP64, KF_FP64_UPDATE): on device arrays with the shape lc, and
+// on host arrays with a grid of that many 256-thread CTAs.
+cudaError_t launch_direct_f64(int kind, int precision, const StepArgs &a,
+                              const cudaLaunchConfig_t &lc);
+void launch_strided_f64(int kind, int precision, const StepArgs &a, unsigned grid,
+                        cudaStream_t s);
+
 // Second pass of KF_ADAPTIVE: redo in FP64 every track whose status the
 // step kernel marked with kRedo (those tracks' outputs are not yet written).
 int launch_redo_pass(int kind, const StepArgs &a, cudaStream_t s);
