@@ -17,8 +17,13 @@
 //  * the transport C' = J C J^T through J's factored form J = J_s + u (ds/dp)
 //    (89 multiply-adds for a cylinder, 70 for a plane), and the update
 //    without the columns and products the general form spends on them.
-// Every operation is a correctly rounded double operation, none is done in
-// less: the seeds only choose where the double iteration starts.
+// Sums, products and fused multiply-adds are correctly rounded double operations
+// and none is done in less: the seeds only choose where the double iteration
+// starts.  1/x and sqrt(x) come out correctly rounded but for a few near-ties,
+// 1/sqrt(x) within 1 ulp; sin and cos carry the table's and two sums' roundings;
+// a quotient is a product with the reciprocal, within 1 ulp (correctly rounded
+// quotients for the arc and S(h) change a whole step's rms error against
+// quadruple precision by less than 1 %).
 //
 // Every rounding is written out (as in kf_num.cuh), so all kernels that call
 // these functions agree bit for bit.
@@ -138,14 +143,19 @@ __device__ __forceinline__ double rsqrt(double x) {
   return fma(mul(y, e), fma(e, 0.375, 0.5), y);
 }
 
-// sqrt(x) = x / sqrt(x): the same with g = x y in front.
+// sqrt(x) = g (1 - e)^(-1/2) with g = x y and e as above.  t = y (x - g^2) is
+// g e and undoes g's own rounding, so the result is the correctly rounded root
+// but for arguments within 2^-20 ulp of a tie (e from g y leaves half of that
+// rounding: 0.75 ulp).  A float's digits are enough for the e beside 1/2.
+// |x| within 2^-60 .. 2^60, where x - g^2 is a normal float.
 __device__ __forceinline__ double sqrt(double x) {
-  if (__double2hiint(x) < 0 || !seedable(x)) return sqrt_any(x);
+  if ((unsigned)__double2hiint(x) - 0x3c300000u >= 0x07800000u) return sqrt_any(x);
   float s;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(cut_normal(x)));
   const double y = from_normal(s), g = mul(x, y);
-  const double e = fma(-g, y, 1.0);
-  return fma(mul(g, e), fma(e, 0.375, 0.5), g);
+  const double d = fma(-g, g, x);
+  const double e = from_normal(__fmul_rn(__fmul_rn(cut(d), s), s));  // 2^-127 for 0
+  return fma(mul(y, d), fma(e, 0.375, 0.5), g);
 }
 
 // ------------------------------------------------------------- sin and cos
