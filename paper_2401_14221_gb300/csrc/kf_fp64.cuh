@@ -271,7 +271,10 @@ static __device__ __noinline__ double atan2_any(double y, double x) { return ::a
 // 0.0123: the next term is 2e-17 of it).  9 FP64 instructions; the library's
 // atan2 takes 45, a correction of atan2f through sincos 16.
 __device__ __forceinline__ double angle(double y, double x, double sh, double ch) {
-  if (top(y) >= 0x46300000u || top(x) >= 0x46300000u) return atan2_any(y, x);  // 2^100, NaN
+  // the larger operand within 2^-100 .. 2^100 (a float cuts the other to zero
+  // only where the angle to an axis is below 2^-26), no NaN; else the library's
+  const unsigned m = top(y) > top(x) ? top(y) : top(x);
+  if (m - 0x39b00000u >= 0x0c800000u) return atan2_any(y, x);
   const float kf = rintf(atan2f(cut(y), cut(x)) * 40.743665431525206f);
   const double k = from_float(kf);
   const sc t = table_entry((int)kf);

@@ -169,6 +169,12 @@ def test_angle(lib, scale):
     assert np.all(err[small] <= U * 8 * np.abs(want[small]))
 
 
+@pytest.mark.parametrize("scale", [-125, -140, -300], ids=str)
+def test_angle_of_tiny_operands(lib, scale):
+    # below the range of a float, where the table angle cannot come from floats
+    test_angle(lib, scale)
+
+
 def test_sinc(lib):
     h = np.concatenate([wide(200000, -40, 1.6, 8), np.linspace(0.0499, 0.0501, 1001)])
     S, dS = call(lib, 6, h)
