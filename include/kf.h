@@ -418,7 +418,10 @@ int kf_propagate_update_host_noalloc(int32_t kind, const kf_params *params,
  * kernel with 1, 2 or 3 CTAs per
  * SM (3: two pipeline stages per CTA instead of three, FP32-arithmetic
  * variants only; the others run it as 2).
- * Chain candidates: 64, 128 or 256 threads per CTA.
+ * Chain candidates: 64, 128 or 256 threads per CTA; a KF_FP64 chain of up to
+ * 96 tracks per SM has one shape (four warps of a 128-thread CTA share 32
+ * tracks), whatever the cache holds: kf_autotune_chain times and returns it and
+ * stores nothing.
  */
 typedef struct {
     int32_t step_kernel;  /* KF_STEP_DIRECT or KF_STEP_STAGED               */

@@ -214,6 +214,11 @@ int launch_chain_adaptive(ChainArgs &a, unsigned blocks, int threads, int dev, i
 }
 
 }  // namespace
+
+bool chain_shares_warps(int precision, int64_t n, int sms) {
+  return precision == KF_FP64 && n <= (int64_t)sms * kGroupTracksPerSm;
+}
+
 }  // namespace kf
 
 extern "C" int kf_set_chain_redo(int32_t mode) {
@@ -278,6 +283,11 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   int dev = 0, sms = 0;
   if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
   if (int rc = staged::sm_count(dev, &sms)) return rc;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (chain_shares_warps(params->precision, d.n, sms)) {
+    chain_group_kernel<<<(unsigned)((d.n + 31) / 32), f64::kGroupThreads, 0, s>>>(a);
+    return check_cuda(cudaGetLastError(), "chain launch");
+  }
   // CTA size: 64 threads spread a small batch over the SMs and waste least in
   // the last wave (us with 64, 128, 256 threads: FP32 5,000 tracks 15.0, 15.0,
   // 17.1, 440,000: 107, 107, 111; FP64 update 60,000: 144, 160, 160; KF_FP64
@@ -295,11 +305,6 @@ extern "C" int kf_kalman_chain(const kf_params *params, kf_layout layout, float 
   const int threads = (cfg.threads == 128 || cfg.threads == 64) ? cfg.threads : 256;
   const int64_t blocks = (d.n + threads - 1) / threads;
   if (blocks > 0x7fffffffLL) return set_error(KF_ERR_ARG, "n too large for one launch");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (params->precision == KF_FP64 && d.n <= (int64_t)sms * kGroupTracksPerSm) {
-    chain_group_kernel<<<(unsigned)((d.n + 31) / 32), f64::kGroupThreads, 0, s>>>(a);
-    return check_cuda(cudaGetLastError(), "chain launch");
-  }
   const unsigned g = (unsigned)blocks;
   int rc = KF_OK;
   switch (params->precision) {

@@ -22,11 +22,12 @@
 
 #include "kf_chain.cuh"
 #include "kf_device.cuh"
+#include "kf_step.cuh"
 
 namespace kf {
 namespace f64 {
 
-constexpr int kGroupThreads = 128;
+constexpr int kGroupThreads = kSharedChainThreads;
 // Of a block's marked tracks, up to this many run 32 at a time by its four
 // warps, more one to a thread: that keeps the schedulers as busy with a seventh
 // fewer instructions.

@@ -128,6 +128,11 @@ int launch_step_staged(int kind, int precision, const StepArgs &a, cudaStream_t 
 // Process-wide choice between the kernels: KF_STEP_AUTO / _DIRECT / _STAGED.
 int step_kernel_mode();
 
+// Whether a chain of n tracks runs with four warps to 32 tracks on a device of
+// that many SMs: one launch shape, kSharedChainThreads a CTA, nothing to tune.
+constexpr int kSharedChainThreads = 128;
+bool chain_shares_warps(int precision, int64_t n, int sms);
+
 // ------------------------------------------------------------- tuning
 enum TuneOp : int { kOpStep = 0, kOpChain = 1 };
 

@@ -6,10 +6,13 @@
 // Candidates.  Single step: the one-thread-per-track kernel with 128 or 256
 // threads per CTA, and (AoSoA layouts, or SoA with n a multiple of 4) the
 // persistent staged kernel with one, two or three CTAs per SM.  Chain: 64,
-// 128 or 256 threads per CTA.  n buckets are
-// powers of two (floor(log2 n)), so one measurement serves batches of
-// similar size.  The cache lives in host memory for the life of the process;
-// kf_autotune_export / kf_autotune_import move it between processes as text.
+// 128 or 256 threads per CTA, or the one shape of a chain whose tracks are
+// shared by four warps (chain_shares_warps), which is timed and reported but
+// not cached: its bucket may reach sizes that run one thread per track.
+// n buckets are powers of two (floor(log2 n)), so one measurement serves
+// batches of similar size.  The cache lives in host memory for the life of the
+// process; kf_autotune_export / kf_autotune_import move it between processes as
+// text.
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -26,6 +29,12 @@
 #include "kf_step.cuh"
 
 namespace kf {
+
+namespace staged {
+// defined with the staged step kernel's dispatch (kf_step_staged.cu)
+int sm_count(int dev, int *out);
+}  // namespace staged
+
 namespace {
 
 thread_local const LaunchConfig *t_override = nullptr;
@@ -199,8 +208,14 @@ extern "C" int kf_autotune_chain(const kf_params *params, kf_layout layout, floa
     return check_cuda(cudaMemcpyAsync(cov, cov_scratch, b21, cudaMemcpyDeviceToDevice, s),
                       "restore covariance");
   };
-  LaunchConfig cands[3] = {{KF_STEP_DIRECT, 64, 0}, {KF_STEP_DIRECT, 128, 0},
+  int dev = 0, sms = 0;
+  if (int rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
+  if (int rc = staged::sm_count(dev, &sms)) return rc;
+  const bool shared = chain_shares_warps(params->precision, d.n, sms);
+  LaunchConfig cands[3] = {{KF_STEP_DIRECT, shared ? kSharedChainThreads : 64, 0},
+                           {KF_STEP_DIRECT, 128, 0},
                            {KF_STEP_DIRECT, 256, 0}};
+  const int ncand = shared ? 1 : 3;
   cudaEvent_t a, b;
   if (int rc = check_cuda(cudaEventCreate(&a), "cudaEventCreate")) return rc;
   if (int rc = check_cuda(cudaEventCreate(&b), "cudaEventCreate")) {
@@ -209,7 +224,7 @@ extern "C" int kf_autotune_chain(const kf_params *params, kf_layout layout, floa
   }
   int rc = KF_OK, best = -1;
   float best_ms = 0.0f;
-  for (int c = 0; rc == KF_OK && c < 3; ++c) {
+  for (int c = 0; rc == KF_OK && c < ncand; ++c) {
     set_thread_override(&cands[c]);
     float total = 0.0f;
     for (int rep = 0; rc == KF_OK && rep < 4; ++rep) {  // rep 0 warms up
@@ -235,7 +250,7 @@ extern "C" int kf_autotune_chain(const kf_params *params, kf_layout layout, floa
   if (rc == KF_OK) rc = restore();
   if (rc == KF_OK) rc = check_cuda(cudaStreamSynchronize(s), "cudaStreamSynchronize");
   if (rc) return rc;
-  tune_store(kOpChain, 0, params->precision, d.soa, d.lw, d.n, cands[best], best_ms);
+  if (!shared) tune_store(kOpChain, 0, params->precision, d.soa, d.lw, d.n, cands[best], best_ms);
   out->step_kernel = cands[best].kernel;
   out->threads = cands[best].threads;
   out->ctas_per_sm = cands[best].ctas_per_sm;
