@@ -71,22 +71,23 @@ __device__ __forceinline__ void redo_track_fp64(const StepArgs &a, int64_t i) {
 // The redo pass of KF_ADAPTIVE: each block gathers the marked tracks of its
 // span of kRedoSpan tracks (one 16-byte status load per 16 tracks), then its
 // threads run the FP64 step on them, one each.  (Four warps sharing 32 tracks,
-// as in the chain's redo, does not pay for one step: with 2,048-track spans
-// 300,007 tracks took 30.3 against 26.4 us, 20,000 17.5 against 18.8.)
-template <int KIND>
-__global__ void __launch_bounds__(kRedoThreads)
+// as in the chain's redo, in the same kernel and with 2,048-track spans, took
+// 7 % off a step of 20,000 tracks and added 15 % to one of 300,007.)  Blocks of
+// THREADS: from kRedoWideTracks on, where the blocks of kRedoThreads no longer
+// fit the device at once (three to an SM), half as many threads (us per step
+// with 64 and 128 threads, 1.92 M tracks with nothing marked p2z 67.0 and 68.3,
+// p2r 71.2 and 72.1, with 0.3 % marked 88 and 94, 99 and 107, with 3 % 157 and
+// 151, 195 and 191; before the line 64 lose: 1.6 M with 0.3 % 76 and 72, 87
+// and 79, with 3 % 141 and 125, 177 and 150).
+constexpr int64_t kRedoWideTracks = 3 * 152 * kRedoSpan;
+template <int KIND, int THREADS>
+__global__ void __launch_bounds__(THREADS)
     redo_pass_kernel(const __grid_constant__ StepArgs a) {
   __shared__ uint16_t list[kRedoSpan];
   __shared__ int count;
-  // Launched as a programmatic dependent of the step kernel: wait here until
-  // it has completed and its status marks are visible.  Before that, let the
-  // next kernel on the stream be scheduled (a staged step then sets up and
-  // prefetches while this pass runs; it waits for this grid to complete
-  // before it reads or writes anything).
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  redo_wait(a.n);
   const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
-  const int cnt = gather_marked<kRedoSpan, kRedoThreads>(a.status, span0, a.n, list, &count);
+  const int cnt = gather_marked<kRedoSpan, THREADS>(a.status, span0, a.n, list, &count);
   for (int q = threadIdx.x; q < cnt; q += blockDim.x) redo_track_fp64<KIND>(a, span0 + list[q]);
 }
 
@@ -98,15 +99,21 @@ int launch_redo_pass(int kind, const StepArgs &a, cudaStream_t s) {
   // programmatic dependent launch: scheduled while the step kernel drains
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(g);
-  cfg.blockDim = dim3(kRedoThreads);
+  const bool wide = a.n <= kRedoWideTracks;
+  cfg.blockDim = dim3(wide ? kRedoThreads : 64);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = kind == kP2z ? cudaLaunchKernelEx(&cfg, redo_pass_kernel<kP2z>, a)
-                                     : cudaLaunchKernelEx(&cfg, redo_pass_kernel<kP2r>, a);
+  cudaError_t e;
+  if (kind == kP2z)
+    e = wide ? cudaLaunchKernelEx(&cfg, redo_pass_kernel<kP2z, kRedoThreads>, a)
+             : cudaLaunchKernelEx(&cfg, redo_pass_kernel<kP2z, 64>, a);
+  else
+    e = wide ? cudaLaunchKernelEx(&cfg, redo_pass_kernel<kP2r, kRedoThreads>, a)
+             : cudaLaunchKernelEx(&cfg, redo_pass_kernel<kP2r, 64>, a);
   return check_cuda(e, "adaptive redo pass launch");
 }
 

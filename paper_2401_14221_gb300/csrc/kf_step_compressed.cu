@@ -113,17 +113,23 @@ __global__ void __launch_bounds__(256)
 
 // KF_ADAPTIVE's second pass on the compressed store: tracks marked kRedo
 // are decoded again from their (untouched) inputs and stepped in FP64.  Each
-// block gathers the marked tracks of its span first, so warps run full.
-template <int KIND>
-__global__ void __launch_bounds__(kRedoThreads)
+// block gathers the marked tracks of its span first, so warps run full.  Blocks
+// of THREADS: up to kRedoWideTracks as for the FP32 store; beyond it, where two
+// spans come to an SM, half as many threads leave the next staged step's blocks
+// their registers (us per step with 64 and 128 threads: 960,000 tracks with
+// nothing marked p2z 30.1 and 30.8, p2r 34.5 and 35.2, with 0.3 % marked 44.9
+// and 44.2, 53.3 and 53.1, with 3 % 79 and 86, 105 and 109; 1.92 M with nothing
+// marked 64.5 and 67.7, 62.0 and 63.0, with 0.3 % 81 and 87, 88 and 98; but
+// 640,000 with 3 % 65 and 60, 101 and 78).
+constexpr int64_t kRedoWideTracks = 192 * kRedoSpan;
+template <int KIND, int THREADS>
+__global__ void __launch_bounds__(THREADS)
     redo_compressed_kernel(const __grid_constant__ CompressedArgs a) {
   __shared__ uint16_t list[kRedoSpan];
   __shared__ int count;
-  // a programmatic dependent of the step kernel, as the FP32-store redo pass
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  redo_wait(a.n);
   const int64_t span0 = (int64_t)blockIdx.x * kRedoSpan;
-  const int cnt = gather_marked<kRedoSpan, kRedoThreads>(a.status, span0, a.n, list, &count);
+  const int cnt = gather_marked<kRedoSpan, THREADS>(a.status, span0, a.n, list, &count);
   for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
     const int64_t i = span0 + list[q];
     const Loc l6 = locate<6>(i, a.n, a.soa, a.lw);
@@ -230,14 +236,20 @@ extern "C" int kf_propagate_update_compressed(
   if (params->precision != KF_ADAPTIVE) return KF_OK;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((d.n + kRedoSpan - 1) / kRedoSpan));
-  cfg.blockDim = dim3(kRedoThreads);  // a block gathers its span of kRedoSpan
+  const bool wide = d.n <= kRedoWideTracks;
+  cfg.blockDim = dim3(wide ? kRedoThreads : 64);  // a block gathers its span of kRedoSpan
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = kind == KF_P2Z ? cudaLaunchKernelEx(&cfg, redo_compressed_kernel<kP2z>, a)
-                                       : cudaLaunchKernelEx(&cfg, redo_compressed_kernel<kP2r>, a);
+  cudaError_t e;
+  if (kind == KF_P2Z)
+    e = wide ? cudaLaunchKernelEx(&cfg, redo_compressed_kernel<kP2z, kRedoThreads>, a)
+             : cudaLaunchKernelEx(&cfg, redo_compressed_kernel<kP2z, 64>, a);
+  else
+    e = wide ? cudaLaunchKernelEx(&cfg, redo_compressed_kernel<kP2r, kRedoThreads>, a)
+             : cudaLaunchKernelEx(&cfg, redo_compressed_kernel<kP2r, 64>, a);
   return check_cuda(e, "compressed redo pass launch");
 }
