@@ -70,8 +70,13 @@ struct Group {
   __device__ __forceinline__ void put_n(int i, int j, double x) const { put(kN + tri(i, j), x); }
 };
 
-// Warps 1 to 3 only (warp 0 is on the turning angle).
-__device__ __forceinline__ void sync_123() { asm volatile("bar.sync 1, 96;" ::: "memory"); }
+// Warps 1 to 3 only (warp 0 is on the turning angle).  bar.sync wants the whole
+// warp at one instruction, and a lane whose reciprocal has no seed has just been
+// in a call of its own: the warp is brought together first.
+__device__ __forceinline__ void sync_123() {
+  __syncwarp();
+  asm volatile("bar.sync 1, 96;" ::: "memory");
+}
 
 // The sine and cosine of an angle that a warp has just updated (slots s, s+1).
 __device__ __forceinline__ void put_sincos(const Group &g, int s, double x) {
