@@ -595,7 +595,8 @@ int kf_server_destroy(kf_server *s);
  *   KF_STEP_AUTO    (default) the autotuner's choice where it has one, else
  *                   the direct kernel in 128-thread CTAs (on GB300 it leads
  *                   or ties the staged kernel from 2,000 to 3.84 M tracks, at
- *                   every layout and for every variant measured);
+ *                   every layout and for every variant measured, but for
+ *                   KF_FP64_UPDATE steps in a row of 30,000 to 90,000 tracks);
  *   KF_STEP_DIRECT  one thread per track with direct global loads (any
  *                   layout), 128-thread CTAs;
  *   KF_STEP_STAGED  a persistent kernel in which a producer warp streams

@@ -474,7 +474,7 @@ __device__ __forceinline__ void kalman_update_body(T (&p)[6], T (&C)[21], const 
 // the measured columns are K V (C'' H^T = K V cancels no digits), which needs
 // no S^-1 V: 73 FP64 instructions a p2r track where the conversions, two
 // library divisions and the U (S^-1 V) form took about 145 (960,000 p2r
-// tracks 250 -> 134 us).
+// tracks 250 -> 130 us).
 template <int SKIP, int M1, bool UNIT0>
 __device__ __forceinline__ bool kalman_update_f64(float (&p)[6], float (&C)[21],
                                                   const float (&U0f)[6], const float (&U1f)[6],

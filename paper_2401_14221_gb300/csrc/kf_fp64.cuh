@@ -610,7 +610,7 @@ __device__ __forceinline__ unsigned p2z_step(double (&p)[6], double (&C)[21], do
 // with the hit's azimuth and z.  p and C are left alone when the track starts
 // outside the cylinder or does not reach it.
 //
-// In the surface frame (Axes) J's rows are t: v, z: e_z + zt e_theta + cz m,
+// In the surface frame (Frame, Slope) J's rows are t: v, z: e_z + zt e_theta + cz m,
 // phi: e_phi + kap e_k + cf m, so C' needs only the two products C m^T and
 // C v^T.
 __device__ __forceinline__ unsigned p2r_step(double (&p)[6], double (&C)[21], double q, double bz,

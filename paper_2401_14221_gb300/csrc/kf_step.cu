@@ -193,12 +193,14 @@ static int launch_step_main(int kind, int precision, const StepArgs &a, cudaStre
   // The staged kernel copies whole tiles of device memory with 16-byte-
   // aligned bulk copies: any AoSoA layout, SoA when n is a multiple of 4.
   const bool staged_ok = !plain_loads && (!a.soa || (a.n & 3) == 0);
-  // The variants bound by the FP64 pipe lead as direct kernels too (direct
-  // against the staged kernel's best shape, AoSoA64).  FP64 update: 1,000,000
-  // tracks p2r 140 and 147 us, p2z 130 and 137; 30,000: 9.6 and 12.5, 9.6 and
-  // 11.5.  KF_FP64 needs 150 registers, which the staged kernel's 96 spill:
-  // 1,000,000 tracks p2r 663 and 681 us, p2z 463 and 464; 30,000: 40 and 50,
-  // 29 and 35; 2,000: 17 and 30, 12 and 21.
+  // The variants bound by the FP64 pipe run as direct kernels too (us, direct
+  // against the staged kernel's best shape, AoSoA64, launches in a row).  FP64
+  // update: 1,000,000 tracks p2r 135 and 146, p2z 126 and 135; 20,000: 9.5 and
+  // 12.0, 8.5 and 11.0.  From 30,000 to 90,000 the staged kernel leads in a row
+  // (60,000: 17.6 and 13.6, 17.1 and 12.5) and loses alone (17 and 19 both), so
+  // the line is left to the tuner.  KF_FP64 needs 157 registers, which the
+  // staged kernel's 96 spill: 1,000,000 tracks p2r 654 and 676, p2z 438 and 457;
+  // 60,000: 54 and 56, 37 and 38; 2,000: 16 and 30, 11 and 21.
   LaunchConfig cfg{KF_STEP_DIRECT, kDirectThreads, 2};
   if (plain_loads) {
     // host or managed memory: the grid-stride kernel below
