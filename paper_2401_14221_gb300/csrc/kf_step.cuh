@@ -62,14 +62,15 @@ constexpr int kRedoThreads = 128;
 // A redo pass is a programmatic dependent of its step: it waits here until that
 // has completed and its status marks are visible.  It lets the next kernel on
 // the stream be scheduled before the wait where the step fills the device (that
-// kernel then sets up and prefetches while this pass runs, and waits for it
-// before it reads or writes anything), after it where step, pass and the next
-// step are on the device together anyway: there the next step's blocks, let in
-// early, keep the pass after them waiting for room.  us per step with nothing
-// marked, before and after the wait: p2z 20,000 tracks 4.24 and 3.45, 50,000
-// 5.83 and 4.04, 100,000 6.44 and 5.32, 200,000 7.88 and 7.62; p2r 500,000
-// 20.47 and 20.83, 960,000 37.4 and 38.4.
-constexpr int64_t kRedoEarlyTracks = 1 << 18;
+// kernel then sets up and asks L2 for its inputs while this pass runs, and waits
+// for it before it reads or writes anything), after it where step, pass and the
+// next step are on the device together anyway: there the next step's blocks, let
+// in early, keep the pass after them waiting for room.  us per step with nothing
+// marked, three batches in turn, before and after the wait: p2z 20,000 tracks
+// 4.22 and 3.40, 60,000 5.76 and 4.49, 100,000 6.68 and 5.45, 130,000 6.95 and
+// 6.27, 200,000 9.31 and 10.36; p2r 60,000 6.19 and 5.11, 130,000 7.50 and 7.43,
+// 200,000 10.4 and 11.8, 960,000 37.4 and 38.4.
+constexpr int64_t kRedoEarlyTracks = 1 << 17;
 __device__ __forceinline__ void redo_wait(int64_t n) {
   const bool early = n > kRedoEarlyTracks;
   if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -64,7 +64,7 @@ def test_step(kind, share):
     fn = kf.kf_p2z_propagate_update if kind == kf.KF_P2Z else kf.kf_p2r_propagate_update
     params = kf.make_params(w.bz, kf.KF_ADAPTIVE)
     compare(lambda lay, outs, status: fn(params, lay, *ins, *outs, *args, status), ins, n,
-            (n - 33 - 4096, 1 << 18))
+            (n - 33 - 4096, 1 << 17))
 
 
 @SHARES
@@ -77,4 +77,4 @@ def test_compressed_step(kind, share):
            kf.to_device_rho(rep(rho), lay, "cuda"))
     params = kf.make_params(w.bz, kf.KF_ADAPTIVE)
     compare(lambda lay, outs, status: kf.kf_propagate_update_compressed(
-        kind, params, lay, *ins, *outs, *args, status), ins, n, (n - 33 - 4096, 1 << 18))
+        kind, params, lay, *ins, *outs, *args, status), ins, n, (n - 33 - 4096, 1 << 17))
